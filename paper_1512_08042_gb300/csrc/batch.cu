@@ -244,9 +244,8 @@ hyb_status hyb_batch_init(const hyb_params* p, int32_t n, void* arena, uint64_t 
         pb[r + 1] = pb[r] + (c.d.ncells + 31) / 32;  // collide blocks of 32 cells
         pb4[r + 1] = pb4[r] + (c.d.ncells + 15) / 16;  // and of 16
         pn[r + 1] = pn[r] + c.d.nnodes;
-        const uint32_t pool = hyb::collide_pool(c, 8), pool4 = hyb::collide_pool(c, 4);
+        const uint32_t pool = hyb::collide_pool(c);
         if (pool > d.pool) d.pool = pool;
-        if (pool4 > d.pool4) d.pool4 = pool4;
         if ((uint32_t)c.d.bin > d.maxbin) d.maxbin = (uint32_t)c.d.bin;
     }
     d.tot_cells = pc[n];

@@ -56,6 +56,24 @@ __device__ __forceinline__ uint32_t rec_tag(const double* rec, int64_t i) {
     return (uint32_t)__double_as_longlong(rec[(int64_t)kRec * i + RS_TAG]);
 }
 
+// R records per lane held in registers, loaded whole (FP32).
+template <typename Real, int R>
+struct Held {};
+template <int R>
+struct Held<float, R> {
+    float4 a[R], b[R];
+    __device__ __forceinline__ void load(const float* rec, int64_t i, int r) {
+        const float4* p = reinterpret_cast<const float4*>(rec + (int64_t)kRec * i);
+        a[r] = p[0];
+        b[r] = p[1];
+    }
+    __device__ __forceinline__ uint32_t key(int r) const { return __float_as_uint(b[r].z); }
+    __device__ __forceinline__ void get(int r, float (&p)[6]) const {  // x y z vx vy vz
+        p[0] = a[r].x, p[1] = a[r].y, p[2] = b[r].y;
+        p[3] = a[r].z, p[4] = a[r].w, p[5] = b[r].x;
+    }
+};
+
 // What a move needs: channel sizes, step constants rounded to the state precision, the key.
 template <typename Real>
 struct MoveCtx {
@@ -175,8 +193,9 @@ __device__ __forceinline__ Real wrap_periodic(Real v, Real period) {
 // wall draws). Returns its new cell of the context, (iz nly + iy - y0) ncx + ix, with dir = -1;
 // for a particle that leaves a streamwise slab, the channel's cell (iz ncy + iy) ncx + ix and
 // dir = 0 (towards lower rows) or 1 (higher rows, across the periodic end included). `key` is
-// its order key in the new cell.
-template <typename Real, bool Z3>
+// its order key in the new cell. SLAB = false: the context holds the whole channel (y0 = 0,
+// nly = ncy), which no particle leaves.
+template <typename Real, bool Z3, bool SLAB = true>
 __device__ __forceinline__ uint32_t move_particle(const MoveCtx<Real>& m, const Origin& o, uint32_t k,
                                                   uint32_t s, Real& px, Real& py, Real& pz, Real& ux,
                                                   Real& uy, Real& uz, uint32_t& hits, uint32_t& caps,
@@ -202,6 +221,10 @@ __device__ __forceinline__ uint32_t move_particle(const MoveCtx<Real>& m, const 
         iz = iz < 0 ? 0 : (iz > m.ncz - 1 ? m.ncz - 1 : iz);
     }
     key = order_key<Real, Z3>(m, o, k, ix, iy, iz);
+    if constexpr (!SLAB) {
+        dir = -1;
+        return (uint32_t)((iz * m.ncy + iy) * m.ncx + ix);
+    }
     const int iyl = iy - m.y0;
     if (iyl >= 0 && iyl < m.nly) {
         dir = -1;

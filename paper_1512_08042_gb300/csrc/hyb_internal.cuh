@@ -197,10 +197,10 @@ __device__ __forceinline__ uint4 philox(uint4 c, uint32_t k0, uint32_t k1) {
             k0 += 0x9E3779B9u;
             k1 += 0xBB67AE85u;
         }
-        const uint32_t lo0 = 0xD2511F53u * c.x;
-        const uint32_t hi0 = __umulhi(0xD2511F53u, c.x);
-        const uint32_t lo1 = 0xCD9E8D57u * c.z;
-        const uint32_t hi1 = __umulhi(0xCD9E8D57u, c.z);
+        // one wide multiplication gives both halves of a product
+        const uint64_t p0 = (uint64_t)0xD2511F53u * c.x, p1 = (uint64_t)0xCD9E8D57u * c.z;
+        const uint32_t lo0 = (uint32_t)p0, hi0 = (uint32_t)(p0 >> 32);
+        const uint32_t lo1 = (uint32_t)p1, hi1 = (uint32_t)(p1 >> 32);
         c = make_uint4(hi1 ^ c.y ^ k0, lo1, hi0 ^ c.w ^ k1, lo0);
     }
     return c;
@@ -552,8 +552,7 @@ struct BatchDev {
     const int64_t* pre_d2l = nullptr;
     const int64_t* pre_l2d = nullptr;
     int64_t tot_cells = 0, tot_blocks = 0, tot_blocks4 = 0, tot_nodes = 0, tot_d2l = 0, tot_l2d = 0;
-    // collide shared-memory pools of 32- and 16-cell blocks: the largest over the replicas
-    uint32_t pool = 0, pool4 = 0;
+    uint32_t pool = 0;    // collide shared-memory pool of a warp: the largest over the replicas
     uint32_t maxbin = 0;  // the largest bin over the replicas (the collide's key bitmaps)
     // threads per block of each tuned class (the collide: 256 for 32 cells, 128 for 16)
     int move_block = 256, lbm_block = 128, d2l_block = 128, collide_block = 256;
@@ -564,7 +563,7 @@ size_t lbm_args_bytes(int real_bytes);
 void lbm_args_fill(Ctx& c, int cur_f, void* out);
 size_t map_args_bytes(int real_bytes);
 void map_args_fill(Ctx& c, int cur_p, int cur_f, const int32_t* list, int32_t n, void* out);
-uint32_t collide_pool(const Ctx& c, int warps = 8);
+uint32_t collide_pool(const Ctx& c);
 cudaError_t launch_batch_move(BatchDev& b, int cur_p);
 cudaError_t launch_batch_collide(BatchDev& b, int cur_p);
 cudaError_t launch_batch_lbm(BatchDev& b, int cur_f);

@@ -11,13 +11,12 @@
 //              order key (its displacement's neighbour offset, then its rank in the old cell;
 //              see order_key) are appended to the bin of its new cell in half p^1 by a
 //              warp-aggregated atomic.
-//   k_collide  32 consecutive cells per block, a group of 8 lanes per cell: each arrival's
+//   k_collide  four consecutive cells per warp, a group of 8 lanes per cell: each arrival's
 //              rank by key comes from a bitmap of the cell's keys with prefix counts, each
-//              arrival is placed at its rank in a shared-memory pool, the NTC candidates of
-//              all 32 cells are drawn by the whole
-//              block and applied by one warp with a lane per cell (Eq. collisionnumber), the
-//              sums 1, v, vv, vvv are added to the FP64 cumulative sums of the cell (Sec. 2.1,
-//              Fig. 1) and the sorted cell is written back in place.
+//              arrival is placed at its rank in the warp's shared-memory pool, the NTC candidates
+//              of a cell are drawn and settled eight at a time by its lanes
+//              (Eq. collisionnumber), the sums 1, v, vv, vvv are added to the FP64 cumulative
+//              sums of the cell (Sec. 2.1, Fig. 1) and the sorted cell is written back in place.
 //   k_step_end one thread per context after each collide pass: publishes the particle count
 //              and advances the step and sample counters.
 // Several steps in one call fuse the collide of step s with the move of step s + 1: the
@@ -27,6 +26,7 @@
 // This file is compiled without FMA contraction so that positions, cell keys, pair choices
 // and post-collision velocities are the IEEE float (or double) results of the written
 // expressions.
+#include <cmath>
 #include <cstring>
 
 #include "dsmc_move.cuh"
@@ -225,20 +225,27 @@ __global__ void __launch_bounds__(256, 4) k_move(Launch<DsmcArgs<Real>> L) {
 }
 
 // ---------------------------------------------------------------------------------------
-// Collide: a group of G lanes per cell, 32 / G cells per warp. Every instruction of the
-// serial NTC chain then advances 32 / G cells at once. All loops that contain shuffles have
-// warp-uniform trip counts (groups whose cell has less work are masked), so every shuffle is
-// executed by the full warp.
+// Collide: a warp takes four consecutive cells, eight lanes per cell, from the arrivals to the
+// written or moved particles, without waiting for any other warp. All loops that contain
+// shuffles have warp-uniform trip counts (groups whose cell has less work are masked), so
+// every shuffle is executed by the full warp.
+//
+// Bound by latency and issue, not by bandwidth (ncu, 6.55M particles with Kn along the channel:
+// issue 48%, DRAM 30% of its peak, 16.7 warp instructions per particle). No block barrier: while
+// one warp of a block ran the block's NTC chains and the others waited, barriers were a fifth of
+// the stalls. 20 steps, before and after: 105M particles 78.0 -> 70.3 ms, 819k 2.17 -> 1.50 ms,
+// 3D 6.55M 13.6 -> 9.6 ms, 64 batched channels (10 steps) 1.50 -> 1.19 ms.
 constexpr int kGroup = 8;
+constexpr int kWarpCells = 32 / kGroup;
 
-// A collide block has W warps for 4 W cells (W = 8: 32 cells, the default; W = 4: 16 cells,
-// twice the blocks per SM); its launch bounds keep 80 registers (FP32) or 128 (FP64).
+// Blocks of 8 warps (32 cells) or 4 (16 cells) only group warps for a launch. 24 resident warps
+// per SM in FP32 (80 registers): 20, 28 and 32 warps took 72.6, 75.0 and 90.8 ms for the 105M
+// particles' 20 steps against 70.8 ms, more warps spilling what the held arrivals need.
 constexpr int kCollideWarps = 8;
 template <typename Real, int W>
 struct CollideCfg {
-    static constexpr int MINB = (sizeof(Real) == 4 ? 3 : 2) * 8 / W;  // resident blocks per SM
+    static constexpr int MINB = (sizeof(Real) == 4 ? 24 : 16) / W;  // resident blocks per SM
 };
-constexpr int kChainSteps = 24;   // candidates per cell drawn per pass of the NTC phase
 enum CollideMode : int { MODE_COLLIDE = 0, MODE_FUSED = 1 };
 
 // Real arrays of the shared-memory pool per slot: vx, vy, vz, x, y (, z)
@@ -255,6 +262,17 @@ __host__ __device__ constexpr int bitmap_words(uint32_t bin) {
 }
 // Keys of farther-displaced particles a cell lists for their ranks (more are counted in full).
 constexpr int kFarList = 8;
+
+// Shared memory of one warp: the pool of its cells' particles (pool_reals Real per slot), then
+// its cells' key bitmaps (words, listed far keys, prefix bytes), in whose place the cells'
+// FP64 sums are copied in once the ranks are taken.
+template <typename Real, bool Z3>
+__host__ __device__ constexpr uint32_t collide_warp_smem(uint32_t pool, uint32_t bin) {
+    const uint32_t bits = (uint32_t)kWarpCells * ((uint32_t)bitmap_words<Z3>(bin) * 5u + (kFarList + 1u) * 4u);
+    const uint32_t sums = (uint32_t)kWarpCells * kMoments * 8u;
+    const uint32_t pv = (pool * (uint32_t)(pool_reals<Z3>() * sizeof(Real)) + 15u) / 16u * 16u;
+    return pv + ((bits > sums ? bits : sums) + 15u) / 16u * 16u;
+}
 
 // Adds a particle's velocity moments to a lane's partial sums: u, the six distinct products
 // u_i u_j and the ten distinct u_i u_j u_k, in the order of the sampled sums (mo[0], the count,
@@ -273,380 +291,320 @@ __device__ __forceinline__ void add_moments(Real (&mo)[kMoments], Real ux, Real 
     mo[18] = fma(zz, uy, mo[18]); mo[19] = fma(zz, uz, mo[19]);
 }
 
-// The block of 32 consecutive cells `blk` (of nblk) of one context: the arrivals of half
-// p^1 (d*) are put in stable order, collided and sampled; MODE_COLLIDE writes them back in
-// place, MODE_FUSED moves them on (step s + 1) into the bins of half p (s*), except cells
-// marked in a.coupled, which are written back in place for LB2DSMC.
-template <typename Real, bool Z3, int MODE, int W>
-__device__ __forceinline__ void collide_block(const DsmcArgs<Real>& a, uint32_t pool, int blk) {
+// The NTC candidates of a cell group's cell (nsel of them, n particles, velocities at vx, vy,
+// vz), applied in their order. The cell's lanes draw eight consecutive candidates at a time and
+// settle them together: every pending lane forms its relative speed from the current
+// velocities, the running (sigma c_r)_max up to its candidate by a prefix maximum and its
+// decision; a candidate that shares a particle with an earlier one of the window that collides
+// must see that collision, so the candidates before the first such one are final and the others
+// are taken again from the updated velocities. The results are those of applying the candidates
+// one after another, bit for bit. Shared particles are found with 64-bit sets of the particles
+// (index modulo 64; an alias only takes a candidate again). The first pending candidate is
+// always final, so every pass settles at least one.
+template <typename Real>
+__device__ __forceinline__ void ntc_collisions(uint64_t seed, uint32_t gc, uint32_t s, uint32_t n, uint32_t nsel,
+                                               Real* vx, Real* vy, Real* vz, int grp, int gl, Real& cm,
+                                               uint32_t& ncoll, uint32_t& flags) {
     constexpr int G = kGroup;
-    constexpr int CPW = 32 / G;           // cells per warp in phases A and C
-    constexpr int WARPS = W;
-    constexpr int NC = WARPS * CPW;       // cells per block (one chain lane each in phase B)
-    constexpr int SMALL = 64;             // keys of the first SMALL slots loaded with the count
-    constexpr int R = SMALL / G;
-    constexpr int KC = kChainSteps;       // candidates per cell drawn per pass of phase B
-    constexpr int NR = pool_reals<Z3>();
-    constexpr int SJ = 2;                 // arrivals per lane whose loads are in flight together
-    static_assert(NC <= 32, "phase B runs one lane per cell of the block in one warp");
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    // per cell of the block, by phase B's lanes (lanes past NC are empty cells)
-    __shared__ uint32_t s_n[32], s_off[32], s_nsel[32];
-    __shared__ Real s_cm[32];
-    if (NC < 32 && threadIdx.x >= NC && threadIdx.x < 32) {
-        s_n[threadIdx.x] = 0u;
-        s_nsel[threadIdx.x] = 0u;
-        s_cm[threadIdx.x] = (Real)0;
+    const uint32_t maxsel = __reduce_max_sync(kFull, nsel);
+    for (uint32_t k0 = 0; k0 < maxsel; k0 += G) {
+        const uint32_t k = k0 + (uint32_t)gl;
+        bool pend = k < nsel;
+        uint32_t i = 0, j = 0;
+        Real R = (Real)0, nx = (Real)0, ny = (Real)0, nz = (Real)0;
+        int ok = 0;
+        if (pend) {
+            const uint4 r = draw(seed, gc, s, TAG_NTC_PAIR, k, 0);
+            i = uindex(r.x, n);
+            j = uindex(r.y, n - 1u);
+            if (j >= i) j += 1u;
+            R = (Real)u01f(r.z);
+            ok = unit_vector(seed, gc, s, k, nx, ny, nz);
+        }
+        const uint32_t bi = 1u << (i & 31u), bj = 1u << (j & 31u);
+        const uint32_t mlo = ((i & 32u) ? 0u : bi) | ((j & 32u) ? 0u : bj);
+        const uint32_t mhi = ((i & 32u) ? bi : 0u) | ((j & 32u) ? bj : 0u);
+        while (__any_sync(kFull, pend)) {
+            Real ax = 0, ay = 0, az = 0, bx = 0, by = 0, bz = 0, cr = 0;
+            Real v = cm;
+            if (pend) {
+                ax = vx[i], ay = vy[i], az = vz[i];
+                bx = vx[j], by = vy[j], bz = vz[j];
+                const Real ddx = ax - bx, ddy = ay - by, ddz = az - bz;
+                cr = sqrt(ddx * ddx + ddy * ddy + ddz * ddz);
+                if (cr > cm) v = cr;
+            }
+#pragma unroll
+            for (int o = 1; o < G; o <<= 1) {
+                const Real t = __shfl_up_sync(kFull, v, o, G);
+                if (gl >= o && t > v) v = t;
+            }
+            const bool acc = pend && cr > R * v;
+            const bool coll = acc && ok;
+            uint32_t elo = coll ? mlo : 0u, ehi = coll ? mhi : 0u;
+#pragma unroll
+            for (int o = 1; o < G; o <<= 1) {
+                const uint32_t tl = __shfl_up_sync(kFull, elo, o, G), th = __shfl_up_sync(kFull, ehi, o, G);
+                if (gl >= o) elo |= tl, ehi |= th;
+            }
+            // exclusive: the particles of the earlier lanes' collisions
+            elo = __shfl_up_sync(kFull, elo, 1, G);
+            ehi = __shfl_up_sync(kFull, ehi, 1, G);
+            const bool conf = pend && gl > 0 && ((elo & mlo) | (ehi & mhi)) != 0u;
+            const unsigned cb = (__ballot_sync(kFull, conf) >> (G * grp)) & ((1u << G) - 1u);
+            const int cut = cb ? __ffs((int)cb) - 1 : G;
+            if (pend && gl < cut) {
+                pend = false;
+                if (coll) {
+                    const Real cx = (ax + bx) * (Real)0.5;
+                    const Real cy = (ay + by) * (Real)0.5;
+                    const Real cz = (az + bz) * (Real)0.5;
+                    const Real h = cr * (Real)0.5;
+                    const Real hx = h * nx, hy = h * ny, hz = h * nz;
+                    vx[i] = cx + hx;
+                    vy[i] = cy + hy;
+                    vz[i] = cz + hz;
+                    vx[j] = cx - hx;
+                    vy[j] = cy - hy;
+                    vz[j] = cz - hz;
+                    ncoll += 1;
+                } else if (acc) {
+                    flags |= HYB_ST_SCATTER_CAP;
+                }
+            }
+            cm = __shfl_sync(kFull, v, cut - 1, G);
+            __syncwarp();
+        }
     }
-    __shared__ uint32_t s_fits;
-    __shared__ unsigned long long s_cnt[WARPS][2];
-    __shared__ uint32_t s_live[WARPS], s_flags[WARPS];
-    __shared__ __align__(16) double s_acc[NC][kMoments];
-    const int w = threadIdx.x >> 5;
+}
+
+// The four consecutive cells from cell0 of one context, by one warp: the arrivals of half p^1
+// (d*) are put in stable order, collided and sampled; MODE_COLLIDE writes them back in
+// place, MODE_FUSED moves them on (step s + 1) into the bins of half p (s*), except cells
+// marked in a.coupled, which are written back in place for LB2DSMC. Returns the warp's
+// candidates, collisions, particles and status bits.
+template <typename Real, bool Z3, int MODE>
+__device__ __forceinline__ void collide_warp(const DsmcArgs<Real>& a, uint32_t pool, int cell0, unsigned char* smem,
+                                             uint32_t& ncand, uint32_t& ncoll, uint32_t& nlive,
+                                             uint32_t& flags) {
+    constexpr int G = kGroup;
+    constexpr int NR = pool_reals<Z3>();
+    // FP32: the first SMALL arrivals of a cell are held in registers between the marking of
+    // their keys and their placement (48 or 32 held: 72.2 or 77.4 ms against 70.8 ms, none 80.3 ms,
+    // at 105M particles); FP64 (twice the registers) reads them again
+    constexpr int SMALL = 64;
+    constexpr int R = SMALL / G;
+    constexpr bool HELD = sizeof(Real) == 4;
+    constexpr int SJ = 2;  // arrivals per lane whose loads are in flight together when read again
     const unsigned lane = lane_id();
     const int grp = (int)lane / G, gl = (int)lane % G;
-    const int gi = w * CPW + grp;  // the group's cell within the block
     const uint32_t bin = (uint32_t)a.bin;
-    // shared memory: the block's pool of vx, vy, vz, x, y (, z) (Real), `pool` slots each, then the candidates of one pass of phase B, in the same space as the cells'
-    // key bitmaps of phase A (BW words and BW prefix bytes per cell)
-    Real* pv = reinterpret_cast<Real*>(smem_raw);
-    uint32_t* c_ij = reinterpret_cast<uint32_t*>(pv + NR * (size_t)pool);
+    Real* pv = reinterpret_cast<Real*>(smem);
+    unsigned char* scratch = smem + ((size_t)pool * NR * sizeof(Real) + 15) / 16 * 16;
     const int BW = bitmap_words<Z3>(bin);
     const int CW = (BW + G - 1) / G;
     const uint32_t lim = (uint32_t)BW * 32u;
-    uint32_t* s_bm = c_ij;
-    uint32_t* s_fl = s_bm + NC * BW;
-    uint8_t* s_pf = reinterpret_cast<uint8_t*>(s_fl + NC * (kFarList + 1));
-    Real* c_R = reinterpret_cast<Real*>(c_ij + NC * KC);
-    Real* c_nx = c_R + NC * KC;
-    Real* c_ny = c_nx + NC * KC;
-    Real* c_nz = c_ny + NC * KC;
+    uint32_t* bm = reinterpret_cast<uint32_t*>(scratch) + grp * BW;
+    uint32_t* fl = reinterpret_cast<uint32_t*>(scratch) + kWarpCells * BW + grp * (kFarList + 1);
+    uint8_t* pf = scratch + (size_t)kWarpCells * (BW + kFarList + 1) * 4 + grp * BW;
+    double* sums = reinterpret_cast<double*>(scratch) + grp * kMoments;  // after the ranks
     const uint32_t s = a.ctrl[CTRL_STEP];
     const bool do_sample = (s % (uint32_t)a.sample_every) == 0u;
-    const Real coll_dt = a.coll_r;
-    unsigned long long ncand_tot = 0, ncoll_tot = 0;
-    uint32_t flags = 0, nlive = 0;
     uint32_t hits = 0, caps = 0, lost = 0;
 
-    const int c = blk * NC + gi;
+    const int c = cell0 + grp;
     const bool has = c < a.ncells;
     const int64_t base = (int64_t)c * bin;
     // the channel's cell: the key of the random streams and of the stable order
     const uint32_t gc = global_cell((uint32_t)c, a.ncx, a.ncy, a.y0, a.ncy_g);
     const Real* __restrict__ drec = a.drec;
-    // the cell's loads are issued together: count, the first SMALL keys and the leader's NTC
-    // state
     uint32_t n_all = has ? a.count_d[c] : 0u;
-    // the cell's FP64 sums, copied to shared memory while the block works (10 x 16 bytes)
-    if (has && do_sample)
-        for (int j = gl; j < 2 * kMoments / 4; j += G)
-            cp_async16(&s_acc[gi][2 * j], &a.acc[(size_t)c * kMoments + 2 * j]);
-    cp_async_commit();
-    uint32_t vl[R];
+    // the first half of the held arrivals is read beside the count (a bin has at least 32 slots)
+    Held<Real, R> held;
+    if constexpr (HELD) {
 #pragma unroll
-    for (int r = 0; r < R; ++r) {
-        const uint32_t k = (uint32_t)(gl + G * r);
-        vl[r] = (has && k < bin) ? rec_tag(drec, base + k) : 0xFFFFFFFFu;
+        for (int r = 0; r < R / 2; ++r)
+            if (has) held.load(drec, base + gl + G * r, r);
     }
     uint32_t nb0 = 0;
     Real cm0 = (Real)0, rem0 = (Real)0;
-    if (has && gl == 0) {
+    if (has) {
         nb0 = a.nbar_sum[c];
         cm0 = a.crmax[c];
         rem0 = a.rem[c];
     }
     const bool moving = MODE == MODE_FUSED && has && !(a.coupled && a.coupled[c]);
     if (n_all > bin) n_all = bin;
-    // the cells' regions of the block pool (exclusive scan of the counts); if they do not
-    // fit, the cells take the whole pool one after another
-    if (gl == 0) s_n[gi] = n_all;
-    __syncthreads();
-    if (w == 0) {
-        const uint32_t x = s_n[lane];
-        uint32_t inc = x;
+    if constexpr (HELD) {
 #pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const uint32_t t = __shfl_up_sync(kFull, inc, o);
-            if (lane >= (unsigned)o) inc += t;
-        }
-        s_off[lane] = inc - x;
-        if (lane == 31) s_fits = inc <= pool ? 1u : 0u;
+        for (int r = R / 2; r < R; ++r)
+            if ((uint32_t)(gl + G * r) < n_all) held.load(drec, base + gl + G * r, r);
     }
-    __syncthreads();
-    const bool fits = s_fits != 0u;
-    const int rounds = fits ? 1 : NC;
+    // the cells' regions of the warp's pool (exclusive sums of the counts); if they do not
+    // fit, the cells take the whole pool one after another
+    uint32_t off = 0, tot = 0;
+#pragma unroll
+    for (int q = 0; q < kWarpCells; ++q) {
+        const uint32_t t = __shfl_sync(kFull, n_all, q * G);
+        if (q < grp) off += t;
+        tot += t;
+    }
+    const bool fits = tot <= pool;
+    const int rounds = fits ? 1 : kWarpCells;
+
+    // A. stable order: every arrival's rank among the cell's arrivals by order key. A key
+    // below W bin (a particle from a neighbouring cell) sets bit `key` of the cell's
+    // bitmap, and its rank is the number of set bits below it: the count before its word
+    // (a prefix over the words, kept modulo 256: a queried word holds its own bit, so
+    // the count is below bin) plus those below it within the word. Larger keys follow
+    // all of these, each ranked by counting the larger keys below it (from a list of the
+    // cell's larger keys while they are few, else from the records).
+    auto clear_keys = [&]() {
+        for (int q = gl; q < BW; q += G) bm[q] = 0u;
+        if (gl == 0) fl[0] = 0u;
+        __syncwarp();
+    };
+    auto mark_key = [&](uint32_t t) {
+        if (t < lim) {
+            atomicOr(&bm[t >> 5], 1u << (t & 31u));
+        } else {
+            const uint32_t j = atomicAdd(&fl[0], 1u);
+            if (j < (uint32_t)kFarList) fl[1 + j] = t;
+        }
+    };
+    auto count_keys = [&]() {  // the prefix counts: lane gl owns words [gl CW, gl CW + CW)
+        __syncwarp();
+        const int q0 = gl * CW, q1 = min(q0 + CW, BW);
+        uint32_t mine = 0;
+        for (int q = q0; q < q1; ++q) mine += (uint32_t)__popc(bm[q]);
+        uint32_t inc = mine;
+#pragma unroll
+        for (int o = 1; o < G; o <<= 1) {
+            const uint32_t t = __shfl_up_sync(kFull, inc, o, G);
+            if (gl >= o) inc += t;
+        }
+        uint32_t run = inc - mine;
+        for (int q = q0; q < q1; ++q) {
+            pf[q] = (uint8_t)run;
+            run += (uint32_t)__popc(bm[q]);
+        }
+        __syncwarp();
+    };
+    auto rank_of = [&](uint32_t t, uint32_t n) -> uint32_t {
+        if (t < lim) {
+            const uint32_t q = t >> 5;
+            return (uint32_t)pf[q] + (uint32_t)__popc(bm[q] & ((1u << (t & 31u)) - 1u));
+        }
+        const uint32_t nfar = fl[0];
+        uint32_t rk = n - nfar;
+        if (nfar <= (uint32_t)kFarList) {
+            for (uint32_t m2 = 0; m2 < nfar; ++m2) rk += fl[1 + m2] < t ? 1u : 0u;
+        } else {
+            for (uint32_t m2 = 0; m2 < n; ++m2) {
+                const uint32_t u = rec_tag(drec, base + m2);
+                rk += (u >= lim && u < t) ? 1u : 0u;
+            }
+        }
+        return rk;
+    };
+    auto place = [&](Real* v, uint32_t rk, Real px, Real py, Real pz, Real ux, Real uy, Real uz) {
+        v[rk] = ux;
+        v[pool + rk] = uy;
+        v[2 * pool + rk] = uz;
+        v[3 * pool + rk] = px;
+        v[4 * pool + rk] = py;
+        if constexpr (Z3) v[5 * (size_t)pool + rk] = pz;
+    };
+    // the arrivals from slot k_first on, read (again) from the records
+    auto place_from = [&](Real* v, uint32_t k_first, uint32_t n) {
+        for (uint32_t k0 = k_first; k0 < n; k0 += SJ * G) {
+            Real p[SJ][6];
+            uint32_t t[SJ];
+#pragma unroll
+            for (int j = 0; j < SJ; ++j) {
+                const uint32_t k = k0 + (uint32_t)(gl + G * j);
+                if (k < n) rec_get(drec, base + k, p[j][0], p[j][1], p[j][2], p[j][3], p[j][4], p[j][5], t[j]);
+            }
+#pragma unroll
+            for (int j = 0; j < SJ; ++j) {
+                const uint32_t k = k0 + (uint32_t)(gl + G * j);
+                if (k < n) place(v, rank_of(t[j], n), p[j][0], p[j][1], p[j][2], p[j][3], p[j][4], p[j][5]);
+            }
+        }
+    };
+    constexpr uint32_t K0 = HELD ? (uint32_t)SMALL : 0u;  // arrivals from here on are not held
+    if (fits) {
+        clear_keys();
+        if constexpr (HELD) {
+#pragma unroll
+            for (int r = 0; r < R; ++r)
+                if ((uint32_t)(gl + G * r) < n_all) mark_key(held.key(r));
+        }
+        for (uint32_t k = K0 + gl; k < n_all; k += G) mark_key(rec_tag(drec, base + k));
+        count_keys();
+        if constexpr (HELD) {
+#pragma unroll
+            for (int r = 0; r < R; ++r)
+                if ((uint32_t)(gl + G * r) < n_all) {
+                    Real p[6];
+                    held.get(r, p);
+                    place(pv + off, rank_of(held.key(r), n_all), p[0], p[1], p[2], p[3], p[4], p[5]);
+                }
+        }
+        place_from(pv + off, K0, n_all);
+        __syncwarp();
+    }
     for (int round = 0; round < rounds; ++round) {
-        const bool act = fits || gi == round;
+        const bool act = fits || grp == round;
         const bool has_r = has && act;
         const uint32_t n = act ? n_all : 0u;
-        const uint32_t poff = fits ? s_off[gi] : 0u;
-        Real* vx = pv + poff;
-        Real* vy = pv + pool + poff;
-        Real* vz = pv + 2 * pool + poff;
-        Real* qx = pv + 3 * pool + poff;
-        Real* qy = pv + 4 * pool + poff;
-        Real* qz = pv + 5 * (size_t)pool + poff;  // 3D only
-        // A. stable order: every arrival's rank among the cell's arrivals by order key. A key
-        // below W bin (a particle from a neighbouring cell) sets bit `key` of the cell's
-        // bitmap, and its rank is the number of set bits below it: the count before its word
-        // (a prefix over the words, kept modulo 256: a queried word holds its own bit, so
-        // the count is below bin) plus those below it within the word. Larger keys follow
-        // all of these, each ranked by counting the larger keys below it (from a list of the
-        // cell's larger keys while they are few, else from the records).
-        {
-            uint32_t* bm = s_bm + gi * BW;
-            uint8_t* pf = s_pf + gi * BW;
-            uint32_t* fl = s_fl + gi * (kFarList + 1);  // count, then the first kFarList keys
-            for (int q = gl; q < BW; q += G) bm[q] = 0u;
-            if (gl == 0) fl[0] = 0u;
+        Real* vx = pv + (fits ? off : 0u);
+        Real* vy = vx + pool;
+        Real* vz = vx + 2 * pool;
+        Real* qx = vx + 3 * pool;
+        Real* qy = vx + 4 * pool;
+        Real* qz = vx + 5 * (size_t)pool;  // 3D only
+        if (!fits) {
+            clear_keys();
+            for (uint32_t k = gl; k < n; k += G) mark_key(rec_tag(drec, base + k));
+            count_keys();
+            place_from(vx, 0u, n);
             __syncwarp();
-#pragma unroll
-            for (int r = 0; r < R; ++r) {
-                const uint32_t k = (uint32_t)(gl + G * r);
-                if (k < n) {
-                    const uint32_t t = vl[r];
-                    if (t < lim) {
-                        atomicOr(&bm[t >> 5], 1u << (t & 31u));
-                    } else {
-                        const uint32_t j = atomicAdd(&fl[0], 1u);
-                        if (j < (uint32_t)kFarList) fl[1 + j] = t;
-                    }
-                }
-            }
-            for (uint32_t k = SMALL + gl; k < n; k += G) {
-                const uint32_t t = rec_tag(drec, base + k);
-                if (t < lim) {
-                    atomicOr(&bm[t >> 5], 1u << (t & 31u));
-                } else {
-                    const uint32_t j = atomicAdd(&fl[0], 1u);
-                    if (j < (uint32_t)kFarList) fl[1 + j] = t;
-                }
-            }
-            __syncwarp();
-            // the prefix counts: lane gl owns words [gl CW, gl CW + CW)
-            const int q0 = gl * CW, q1 = min(q0 + CW, BW);
-            uint32_t tot = 0;
-            for (int q = q0; q < q1; ++q) tot += (uint32_t)__popc(bm[q]);
-            uint32_t inc = tot;
-#pragma unroll
-            for (int o = 1; o < G; o <<= 1) {
-                const uint32_t t = __shfl_up_sync(kFull, inc, o, G);
-                if (gl >= o) inc += t;
-            }
-            uint32_t run = inc - tot;
-            for (int q = q0; q < q1; ++q) {
-                pf[q] = (uint8_t)run;
-                run += (uint32_t)__popc(bm[q]);
-            }
-            const uint32_t nfar = fl[0];
-            const uint32_t nnear = n - nfar;
-            __syncwarp();
-            // each arrival goes to the pool slot of its rank (its record carries its key); the
-            // loads of a lane's arrivals can be in flight together
-            for (uint32_t k0 = 0; k0 < n; k0 += SJ * G) {
-                Real p[SJ][6];
-                uint32_t t[SJ];
-#pragma unroll
-                for (int j = 0; j < SJ; ++j) {
-                    const uint32_t k = k0 + (uint32_t)(gl + G * j);
-                    if (k < n) rec_get(drec, base + k, p[j][3], p[j][4], p[j][5], p[j][0], p[j][1], p[j][2], t[j]);
-                }
-#pragma unroll
-                for (int j = 0; j < SJ; ++j) {
-                    const uint32_t k = k0 + (uint32_t)(gl + G * j);
-                    if (k < n) {
-                        uint32_t rk;
-                        if (t[j] < lim) {
-                            const uint32_t q = t[j] >> 5;
-                            rk = (uint32_t)pf[q] + (uint32_t)__popc(bm[q] & ((1u << (t[j] & 31u)) - 1u));
-                        } else if (nfar <= (uint32_t)kFarList) {
-                            rk = nnear;
-                            for (uint32_t m2 = 0; m2 < nfar; ++m2) rk += fl[1 + m2] < t[j] ? 1u : 0u;
-                        } else {
-                            rk = nnear;
-                            for (uint32_t m2 = 0; m2 < n; ++m2) {
-                                const uint32_t u = rec_tag(drec, base + m2);
-                                rk += (u >= lim && u < t[j]) ? 1u : 0u;
-                            }
-                        }
-                        vx[rk] = p[j][0];
-                        vy[rk] = p[j][1];
-                        vz[rk] = p[j][2];
-                        qx[rk] = p[j][3];
-                        qy[rk] = p[j][4];
-                        if constexpr (Z3) qz[rk] = p[j][5];
-                    }
-                }
-            }
         }
-        // N_cand = 1/2 N Nbar F_N (sigma c_r)_max dt / V_c + remainder (group leader)
-        if (gl == 0) {
-            uint32_t nsel = 0;
-            if (has_r) {
-                const uint32_t nb = nb0 + n;
-                a.nbar_sum[c] = nb;
+        // the ranks are taken: the cell's FP64 sums are copied over the bitmaps while the cell
+        // is collided (10 x 16 bytes)
+        if (has_r && do_sample)
+            for (int j = gl; j < kMoments / 2; j += G)
+                cp_async16(&sums[2 * j], &a.acc[(size_t)c * kMoments + 2 * j]);
+        cp_async_commit();
+        // B. N_cand = 1/2 N Nbar F_N (sigma c_r)_max dt / V_c + remainder, and the candidates
+        uint32_t nsel = 0;
+        Real cm = cm0;
+        if (has_r) {
+            const uint32_t nb = nb0 + n;
+            if (gl == 0) a.nbar_sum[c] = nb;
+            if (n >= 2) {
+                const Real nbar = (Real)nb / (Real)(s + 1u);
+                const Real cdt = a.coll_cell ? a.coll_cell[c] : a.coll_r;
+                const Real want = (Real)0.5 * (Real)n * nbar * cm0 * cdt + rem0;
+                const Real fw = floor(want);
+                if (gl == 0) a.rem[c] = want - fw;
+                if (fw > (Real)16777215) {
+                    nsel = 16777215u;
+                    flags |= HYB_ST_CELL_OVERFLOW;
+                } else {
+                    nsel = (uint32_t)fw;
+                }
+            }
+            if (gl == 0) {
                 nlive += n;
-                if (n > 32767u) {
-                    flags |= HYB_ST_CELL_OVERFLOW;  // pair indices are packed in 15 and 16 bits
-                } else if (n >= 2) {
-                    const Real nbar = (Real)nb / (Real)(s + 1u);
-                    const Real cdt = a.coll_cell ? a.coll_cell[c] : coll_dt;
-                    const Real ncand = (Real)0.5 * (Real)n * nbar * cm0 * cdt + rem0;
-                    const Real fl = floor(ncand);
-                    a.rem[c] = ncand - fl;
-                    if (fl > (Real)16777215) {
-                        nsel = 16777215u;
-                        flags |= HYB_ST_CELL_OVERFLOW;
-                    } else {
-                        nsel = (uint32_t)fl;
-                    }
-                }
-                ncand_tot += nsel;
+                ncand += nsel;
             }
-            s_nsel[gi] = nsel;
-            s_cm[gi] = cm0;
         }
-        __syncthreads();
-        // B. NTC collisions. The candidates of all cells are drawn in parallel by the whole
-        // block, then warp 0 applies them in order, one lane per cell. If the block's
-        // candidates fit the candidate buffer they are packed (cell g at the exclusive scan
-        // of the counts) and drawn in one pass; otherwise every pass draws up to KC
-        // candidates per cell.
-        const uint32_t my_sel = s_nsel[lane];
-        uint32_t sel_inc = my_sel;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const uint32_t t = __shfl_up_sync(kFull, sel_inc, o);
-            if (lane >= (unsigned)o) sel_inc += t;
-        }
-        const uint32_t sel_total = __shfl_sync(kFull, sel_inc, 31);
-        const bool packed = sel_total <= (uint32_t)(NC * KC);
-        const uint32_t maxsel = __reduce_max_sync(kFull, my_sel);
-        const uint32_t npass = packed ? (sel_total > 0u ? 1u : 0u) : (maxsel + KC - 1) / KC;
-        const int tend = packed ? (int)sel_total : NC * KC;
-        Real cm = (Real)0;
-        uint32_t ncoll = 0;
-        Real* gvx = nullptr;
-        Real* gvy = nullptr;
-        Real* gvz = nullptr;
-        if (w == 0) {
-            cm = s_cm[lane];
-            const uint32_t go = fits ? s_off[lane] : 0u;
-            gvx = pv + go;
-            gvy = pv + pool + go;
-            gvz = pv + 2 * pool + go;
-        }
-        for (uint32_t pass = 0; pass < npass; ++pass) {
-            const uint32_t k0 = pass * (uint32_t)KC;
-            for (int tb = w * 32; tb < tend; tb += WARPS * 32) {  // warp-uniform trip count
-                const int t = tb + (int)lane;
-                int g;
-                uint32_t k;
-                bool valid;
-                if (packed) {
-                    // the cell whose range holds slot t: the number of cells whose inclusive
-                    // count is <= t
-                    int lo = 0;
-#pragma unroll
-                    for (int step = 16; step >= 1; step >>= 1) {
-                        const uint32_t v = __shfl_sync(kFull, sel_inc, lo + step - 1);
-                        if (v <= (uint32_t)t) lo += step;
-                    }
-                    g = lo;
-                    const uint32_t ginc = __shfl_sync(kFull, sel_inc, g);
-                    const uint32_t gsel = __shfl_sync(kFull, my_sel, g);
-                    k = (uint32_t)t - (ginc - gsel);
-                    valid = t < tend;
-                } else {
-                    g = t / KC;
-                    k = k0 + (uint32_t)(t % KC);
-                    valid = t < tend && k < s_nsel[g];
-                }
-                if (valid) {
-                    const uint32_t cg = global_cell((uint32_t)(blk * NC + g), a.ncx, a.ncy, a.y0, a.ncy_g);
-                    const uint32_t ng = s_n[g];
-                    const uint4 r = draw(a.seed, cg, s, TAG_NTC_PAIR, k, 0);
-                    const uint32_t ci = uindex(r.x, ng);
-                    uint32_t cj = uindex(r.y, ng - 1u);
-                    if (cj >= ci) cj += 1u;
-                    Real nx = (Real)0, ny = (Real)0, nz = (Real)0;
-                    const int ok = unit_vector(a.seed, cg, s, k, nx, ny, nz);
-                    c_ij[t] = ci | (cj << 15) | (ok ? 0u : 0x80000000u);
-                    c_R[t] = (Real)u01f(r.z);
-                    c_nx[t] = nx;
-                    c_ny[t] = ny;
-                    c_nz[t] = nz;
-                }
-            }
-            __syncthreads();
-            if (w == 0) {
-                // the candidates of this pass for the lane's cell; the particles of the next
-                // candidate are loaded before this one is applied, and taken from registers
-                // where this one changes them
-                const int kend = packed ? (int)my_sel
-                                        : (my_sel > k0 ? (int)min(my_sel - k0, (uint32_t)KC) : 0);
-                const int t0 = packed ? (int)(sel_inc - my_sel) : (int)lane * KC;
-                uint32_t ijn = 0;
-                Real nax = 0, nay = 0, naz = 0, nbx = 0, nby = 0, nbz = 0;
-                if (kend > 0) {
-                    ijn = c_ij[t0];
-                    const uint32_t i = ijn & 0x7FFFu, j = (ijn >> 15) & 0xFFFFu;
-                    nax = gvx[i], nay = gvy[i], naz = gvz[i];
-                    nbx = gvx[j], nby = gvy[j], nbz = gvz[j];
-                }
-#pragma unroll 1
-                for (int kk = 0; kk < kend; ++kk) {
-                    const int t = t0 + kk;
-                    const uint32_t ij = ijn;
-                    const uint32_t i = ij & 0x7FFFu, j = (ij >> 15) & 0xFFFFu;
-                    const Real ax = nax, ay = nay, az = naz;
-                    const Real bx = nbx, by = nby, bz = nbz;
-                    uint32_t in_ = 0xFFFFFFFFu, jn = 0xFFFFFFFFu;
-                    if (kk + 1 < kend) {
-                        ijn = c_ij[t + 1];
-                        in_ = ijn & 0x7FFFu;
-                        jn = (ijn >> 15) & 0xFFFFu;
-                        nax = gvx[in_], nay = gvy[in_], naz = gvz[in_];
-                        nbx = gvx[jn], nby = gvy[jn], nbz = gvz[jn];
-                    }
-                    const Real ddx = ax - bx, ddy = ay - by, ddz = az - bz;
-                    const Real cr = sqrt(ddx * ddx + ddy * ddy + ddz * ddz);
-                    if (cr > cm) cm = cr;
-                    if (cr > c_R[t] * cm) {
-                        if (ij & 0x80000000u) {
-                            flags |= HYB_ST_SCATTER_CAP;
-                        } else {
-                            const Real cx = (ax + bx) * (Real)0.5;
-                            const Real cy = (ay + by) * (Real)0.5;
-                            const Real cz = (az + bz) * (Real)0.5;
-                            const Real h = cr * (Real)0.5;
-                            const Real hx = h * c_nx[t], hy = h * c_ny[t], hz = h * c_nz[t];
-                            const Real pix = cx + hx, piy = cy + hy, piz = cz + hz;
-                            const Real pjx = cx - hx, pjy = cy - hy, pjz = cz - hz;
-                            gvx[i] = pix;
-                            gvy[i] = piy;
-                            gvz[i] = piz;
-                            gvx[j] = pjx;
-                            gvy[j] = pjy;
-                            gvz[j] = pjz;
-                            ncoll += 1;
-                            if (in_ == i) nax = pix, nay = piy, naz = piz;
-                            if (in_ == j) nax = pjx, nay = pjy, naz = pjz;
-                            if (jn == i) nbx = pix, nby = piy, nbz = piz;
-                            if (jn == j) nbx = pjx, nby = pjy, nbz = pjz;
-                        }
-                    }
-                }
-            }
-            __syncthreads();
-        }
-        if (w == 0) {
-            const int cl = blk * NC + (int)lane;
-            if ((int)lane < NC && cl < a.ncells && (fits || (int)lane == round)) a.crmax[cl] = cm;
-            ncoll_tot += ncoll;
-        }
+        ntc_collisions(a.seed, gc, s, n, nsel, vx, vy, vz, grp, gl, cm, ncoll, flags);
+        if (has_r && gl == 0) a.crmax[c] = cm;
         // C. moment sums of the collided particles; the cell is written back in place in
-        // stable order (the collide, and cells the step's LB2DSMC regenerates), or moved on
+        // stable order (the collide, and cells the step's LB2DSMC regenerates), or moved on.
         // Every lane sums its particles gl, gl + G, gl + 2 G, ... in this order, whether in
         // the loop below (cells written back) or in the move (cells moved on), so that the
         // sums of a fused pass equal those of single steps bit for bit.
@@ -679,20 +637,16 @@ __device__ __forceinline__ void collide_block(const DsmcArgs<Real>& a, uint32_t 
                 }
                 uint32_t key1 = 0, ok1 = 0;
                 int dir1 = -1;
-                if (act1)
-                    key1 = move_particle<Real, Z3>(m, org, k1, s + 1u, p1[0], p1[1], p1[2], p1[3], p1[4],
-                                                   p1[5], hits, caps, dir1, ok1);
-                const bool loc1 = act1 && dir1 < 0;
-                const uint32_t arr1 = bin_arrival1(dst.count, key1, loc1, lane);
-                if (loc1) {
+                if (act1)  // (multi-step calls run on whole channels: no particle leaves)
+                    key1 = move_particle<Real, Z3, false>(m, org, k1, s + 1u, p1[0], p1[1], p1[2], p1[3], p1[4],
+                                                          p1[5], hits, caps, dir1, ok1);
+                const uint32_t arr1 = bin_arrival1(dst.count, key1, act1, lane);
+                if (act1) {
                     if (arr1 < bin)
                         put_particle<Real, Z3>(dst, (int64_t)key1 * bin + arr1, ok1, p1[0], p1[1], p1[2],
                                                p1[3], p1[4], p1[5]);
                     else
                         lost += 1;
-                } else if (act1) {
-                    send_particle<Real, Z3>(a.xrec, a.xkey, a.xcount, a.xcap, dir1, key1, ok1, p1[0],
-                                            p1[1], p1[2], p1[3], p1[4], p1[5], lost);
                 }
             }
             // the arrivals of half p^1 are consumed: their count starts the next step's
@@ -716,60 +670,66 @@ __device__ __forceinline__ void collide_block(const DsmcArgs<Real>& a, uint32_t 
                 }
             }
             if (gl == 0) t[0] = (Real)n;  // the particle count, moment 0
+            cp_async_wait_all();
+            __syncwarp();
             if (has_r) {
-                // one FP64 addition per sum to the cell's sums copied in at the block's start
-                // (each sum has one writer per step)
-                cp_async_wait_all();
-                __syncwarp(0xFFu << (8 * grp));
+                // one FP64 addition per sum to the cell's sums copied in above (each sum has
+                // one writer per step)
 #pragma unroll
                 for (int q = 0; q < 3; ++q) {
                     const int mq = 3 * gl + q;
-                    if (mq < kMoments) a.acc[(size_t)c * kMoments + mq] = s_acc[gi][mq] + widen(t[q]);
+                    if (mq < kMoments) a.acc[(size_t)c * kMoments + mq] = sums[mq] + widen(t[q]);
                 }
             }
         }
-        __syncthreads();  // the pool is reused by the next round
+        __syncwarp();  // the pool and the sums are reused by the next round
     }
     if constexpr (MODE == MODE_FUSED) move_events(a.counters, a.ctrl, hits, caps, lost, lane);
-    // event counters: per block, one atomic per counter
-    ncand_tot = __reduce_add_sync(kFull, (unsigned)ncand_tot);
-    ncoll_tot = __reduce_add_sync(kFull, (unsigned)ncoll_tot);
-    nlive = __reduce_add_sync(kFull, nlive);
-    flags = __reduce_or_sync(kFull, flags);
-    if (lane == 0) {
-        s_cnt[w][0] = ncand_tot;
-        s_cnt[w][1] = ncoll_tot;
-        s_live[w] = nlive;
-        s_flags[w] = flags;
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        unsigned long long c0 = 0, c1 = 0;
-        uint32_t nl = 0, fl = 0;
-        for (int v = 0; v < WARPS; ++v) {
-            c0 += s_cnt[v][0];
-            c1 += s_cnt[v][1];
-            nl += s_live[v];
-            fl |= s_flags[v];
-        }
-        if (c0) atomicAdd(&a.counters[HYB_C_CANDIDATES], c0);
-        if (c1) atomicAdd(&a.counters[HYB_C_COLLISIONS], c1);
-        if (nl) atomicAdd(&a.ctrl[CTRL_NACC], nl);
-        if (fl) atomicOr(&a.ctrl[CTRL_STATUS], fl);
-        // (k_step_end, launched after the pass, publishes the count and advances the step: no
-        // block waits here for a grid-wide ticket while it holds its shared memory)
-    }
 }
 
 template <typename Real, bool BATCH, bool Z3 = false, int MODE = MODE_COLLIDE, int W = kCollideWarps>
 __global__ void __launch_bounds__(W * 32, (CollideCfg<Real, W>::MINB))
-    k_collide(Launch<DsmcArgs<Real>> L, uint32_t pool) {
+    k_collide(Launch<DsmcArgs<Real>> L, uint32_t pool, uint32_t warp_smem) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    __shared__ uint32_t s_tot[4], s_done;
+    if (threadIdx.x < 4) s_tot[threadIdx.x] = 0u;
+    if (threadIdx.x == 4) s_done = 0u;
+    __syncthreads();
     pdl_begin();
+    const DsmcArgs<Real>* ap = &L.one;
+    int blk = (int)blockIdx.x;
     if constexpr (BATCH) {
         const int r = replica_of(L.pre, L.nrep, (int64_t)blockIdx.x);
-        collide_block<Real, Z3, MODE, W>(L.tab[r], pool, (int)(blockIdx.x - L.pre[r]));
-    } else {
-        collide_block<Real, Z3, MODE, W>(L.one, pool, (int)blockIdx.x);
+        ap = &L.tab[r];
+        blk = (int)(blockIdx.x - L.pre[r]);
+    }
+    const DsmcArgs<Real>& a = *ap;
+    const int w = threadIdx.x >> 5;
+    uint32_t ncand = 0, ncoll = 0, nlive = 0, flags = 0;
+    const int cell0 = (blk * W + w) * kWarpCells;
+    if (cell0 < a.ncells)
+        collide_warp<Real, Z3, MODE>(a, pool, cell0, smem_raw + (size_t)w * warp_smem, ncand, ncoll, nlive, flags);
+    // event counters: summed over the block in shared memory; the last warp to arrive adds the
+    // block's sums, one atomic per counter (no warp waits for another)
+    ncand = __reduce_add_sync(kFull, ncand);
+    ncoll = __reduce_add_sync(kFull, ncoll);
+    nlive = __reduce_add_sync(kFull, nlive);
+    flags = __reduce_or_sync(kFull, flags);
+    if (lane_id() == 0) {
+        atomicAdd(&s_tot[0], ncand);
+        atomicAdd(&s_tot[1], ncoll);
+        atomicAdd(&s_tot[2], nlive);
+        atomicOr(&s_tot[3], flags);
+        __threadfence_block();
+        if (atomicAdd(&s_done, 1u) == (uint32_t)W - 1u) {
+            __threadfence_block();
+            volatile uint32_t* t = s_tot;
+            if (t[0]) atomicAdd(&a.counters[HYB_C_CANDIDATES], (unsigned long long)t[0]);
+            if (t[1]) atomicAdd(&a.counters[HYB_C_COLLISIONS], (unsigned long long)t[1]);
+            if (t[2]) atomicAdd(&a.ctrl[CTRL_NACC], t[2]);
+            if (t[3]) atomicOr(&a.ctrl[CTRL_STATUS], t[3]);
+            // (k_step_end, launched after the pass, publishes the count and advances the step)
+        }
     }
 }
 
@@ -912,16 +872,6 @@ int grid_for(const Ctx& c, int64_t work, int threads, int per_sm) {
     return (int)g;
 }
 
-// Shared memory of a collide block: the pool (pool_reals Real and one u32 per slot) and one
-// pass of NTC candidates (u32 and 4 Real each).
-template <typename Real, bool Z3, int W = kCollideWarps>
-size_t collide_smem(uint32_t pool, uint32_t bin) {
-    constexpr int NC = W * (32 / kGroup);
-    const size_t cand = (size_t)NC * kChainSteps * (4 + 4 * sizeof(Real));
-    const size_t bits = ((size_t)NC * (bitmap_words<Z3>(bin) * 5 + (kFarList + 1) * 4) + 15) / 16 * 16;
-    return (size_t)pool * (pool_reals<Z3>() * sizeof(Real)) + (cand > bits ? cand : bits);
-}
-
 template <typename Real>
 cudaError_t init_impl(Ctx& c) {
     // the initial particles go to half 0: arguments built with half 1 as the source
@@ -962,9 +912,10 @@ cudaError_t collide_impl_w(Ctx& c, int p) {
     Launch<DsmcArgs<Real>> L{};
     L.one = make_args<Real>(c);
     c.cur_p = save;
-    constexpr int NC = W * (32 / kGroup);
-    const uint32_t pool = collide_pool(c, W);
-    const size_t smem = collide_smem<Real, Z3, W>(pool, (uint32_t)c.d.bin);
+    constexpr int NC = W * kWarpCells;
+    const uint32_t pool = collide_pool(c);
+    const uint32_t warp_smem = collide_warp_smem<Real, Z3>(pool, (uint32_t)c.d.bin);
+    const size_t smem = (size_t)W * warp_smem;
     // (dynamic and static shared memory together may exceed the default 48 KB)
     cudaError_t e = cudaFuncSetAttribute(k_collide<Real, false, Z3, MODE, W>,
                                          cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
@@ -973,7 +924,8 @@ cudaError_t collide_impl_w(Ctx& c, int p) {
     L.total = grid;
     constexpr int kid = MODE == MODE_FUSED ? K_FUSED : K_COLLIDE;
     prof_begin(c, kid);
-    e = launch_pdl(k_collide<Real, false, Z3, MODE, W>, dim3(grid), dim3(W * 32), smem, c.stream, L, pool);
+    e = launch_pdl(k_collide<Real, false, Z3, MODE, W>, dim3(grid), dim3(W * 32), smem, c.stream, L, pool,
+                   warp_smem);
     prof_end(c, kid);
     if (e != cudaSuccess) return e;
     return launch_pdl(k_step_end<Real, false>, dim3(1), dim3(32), 0, c.stream, L);
@@ -1096,21 +1048,21 @@ int collide_per_sm(Kern kernel, int threads, size_t smem) {
 namespace {
 template <int W>
 bool fused_fills_gpu_w(const Ctx& c) {
-    constexpr int NC = W * (32 / kGroup);
-    const uint32_t pool = collide_pool(c, W);
+    constexpr int NC = W * kWarpCells;
+    const uint32_t pool = collide_pool(c);
     const uint32_t bin = (uint32_t)c.d.bin;
     const bool z3 = c.p.ncz >= 2;
     int per_sm;
     if (c.p.real_bytes == 4)
         per_sm = z3 ? collide_per_sm(k_collide<float, false, true, MODE_FUSED, W>, W * 32,
-                                     collide_smem<float, true, W>(pool, bin))
+                                     (size_t)W * collide_warp_smem<float, true>(pool, bin))
                     : collide_per_sm(k_collide<float, false, false, MODE_FUSED, W>, W * 32,
-                                     collide_smem<float, false, W>(pool, bin));
+                                     (size_t)W * collide_warp_smem<float, false>(pool, bin));
     else
         per_sm = z3 ? collide_per_sm(k_collide<double, false, true, MODE_FUSED, W>, W * 32,
-                                     collide_smem<double, true, W>(pool, bin))
+                                     (size_t)W * collide_warp_smem<double, true>(pool, bin))
                     : collide_per_sm(k_collide<double, false, false, MODE_FUSED, W>, W * 32,
-                                     collide_smem<double, false, W>(pool, bin));
+                                     (size_t)W * collide_warp_smem<double, false>(pool, bin));
     if (per_sm < 1) return true;
     const int64_t blocks = (c.d.ncells + NC - 1) / NC;
     return blocks >= (int64_t)per_sm * c.num_sms;
@@ -1121,12 +1073,13 @@ bool dsmc_fused_fills_gpu(const Ctx& c) {
     return c.collide_warps == 4 ? fused_fills_gpu_w<4>(c) : fused_fills_gpu_w<8>(c);
 }
 
-// Pool slots of a collide block of `warps` warps (4 cells each): room for 1.1 ppc per cell on
-// average (the cells' counts add up to about NC ppc with a spread of sqrt(NC ppc); a block
-// whose cells do not fit takes the pool one cell at a time), and at least one full bin.
-uint32_t collide_pool(const Ctx& c, int warps) {
-    const int NC = warps * (32 / kGroup);
-    uint32_t pool = (uint32_t)(((int64_t)NC * c.p.ppc * 11 / 10 + 31) / 32 * 32);
+// Pool slots of a collide warp: its four cells' counts add up to about 4 ppc with a spread of
+// sqrt(4 ppc); room for four such spreads (a warp whose cells do not fit takes the pool one
+// cell at a time), and at least one full bin.
+uint32_t collide_pool(const Ctx& c) {
+    const double mean = (double)kWarpCells * c.p.ppc;
+    uint32_t pool = ((uint32_t)std::ceil(mean + 4.0 * std::sqrt(mean)) + 7u) / 8u * 8u;
+    if (pool > (uint32_t)(kWarpCells * c.d.bin)) pool = (uint32_t)(kWarpCells * c.d.bin);
     if (pool < (uint32_t)c.d.bin) pool = (uint32_t)c.d.bin;
     return pool;
 }
@@ -1150,20 +1103,20 @@ cudaError_t batch_collide_impl(BatchDev& b, int cur_p) {
     L.tab = (const DsmcArgs<Real>*)b.dsmc[cur_p];
     L.nrep = b.nrep;
     cudaError_t e;
+    const uint32_t warp_smem = collide_warp_smem<Real, false>(b.pool, b.maxbin);
+    const size_t smem = (size_t)(b.collide_block / 32) * warp_smem;
     if (b.collide_block == 128) {  // blocks of 16 cells
         L.pre = b.pre_blocks4;
         L.total = b.tot_blocks4;
-        const size_t smem = collide_smem<Real, false, 4>(b.pool4, b.maxbin);
         auto k = k_collide<Real, true, false, MODE_COLLIDE, 4>;
         e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e == cudaSuccess) e = launch_pdl(k, dim3((unsigned)L.total), dim3(128), smem, b.stream, L, b.pool4);
+        if (e == cudaSuccess) e = launch_pdl(k, dim3((unsigned)L.total), dim3(128), smem, b.stream, L, b.pool, warp_smem);
     } else {  // blocks of 32 cells
         L.pre = b.pre_blocks;
         L.total = b.tot_blocks;
-        const size_t smem = collide_smem<Real, false, 8>(b.pool, b.maxbin);
         auto k = k_collide<Real, true, false, MODE_COLLIDE, 8>;
         e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e == cudaSuccess) e = launch_pdl(k, dim3((unsigned)L.total), dim3(256), smem, b.stream, L, b.pool);
+        if (e == cudaSuccess) e = launch_pdl(k, dim3((unsigned)L.total), dim3(256), smem, b.stream, L, b.pool, warp_smem);
     }
     if (e != cudaSuccess) return e;
     return launch_pdl(k_step_end<Real, true>, dim3((unsigned)((L.nrep + 127) / 128)), dim3(128), 0,
