@@ -444,7 +444,7 @@ hyb_status hyb_current(const hyb_ctx* ctx, int32_t* particle_half, int32_t* lb_h
 #define HYB_FUSE_NEVER 2
 hyb_status hyb_set_fuse(hyb_ctx* ctx, int32_t mode);
 
-/* The collide's block shape: 8 warps for 32 cells (the default) or 4 warps for 16 (twice the
+/* The collide's block shape: 4 warps for 16 cells (the default) or 8 warps for 32 (half the
  * blocks per SM; a warp takes four cells in either); HYB_EINVAL for others. The
  * shape changes no result. get returns the shape in use (-1 for a null context).
  * hyb_tune_collide times, for each shape, with and without fusion (HYB_FUSE_ALWAYS,

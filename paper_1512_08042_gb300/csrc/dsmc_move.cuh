@@ -56,24 +56,6 @@ __device__ __forceinline__ uint32_t rec_tag(const double* rec, int64_t i) {
     return (uint32_t)__double_as_longlong(rec[(int64_t)kRec * i + RS_TAG]);
 }
 
-// R records per lane held in registers, loaded whole (FP32).
-template <typename Real, int R>
-struct Held {};
-template <int R>
-struct Held<float, R> {
-    float4 a[R], b[R];
-    __device__ __forceinline__ void load(const float* rec, int64_t i, int r) {
-        const float4* p = reinterpret_cast<const float4*>(rec + (int64_t)kRec * i);
-        a[r] = p[0];
-        b[r] = p[1];
-    }
-    __device__ __forceinline__ uint32_t key(int r) const { return __float_as_uint(b[r].z); }
-    __device__ __forceinline__ void get(int r, float (&p)[6]) const {  // x y z vx vy vz
-        p[0] = a[r].x, p[1] = a[r].y, p[2] = b[r].y;
-        p[3] = a[r].z, p[4] = a[r].w, p[5] = b[r].x;
-    }
-};
-
 // What a move needs: channel sizes, step constants rounded to the state precision, the key.
 template <typename Real>
 struct MoveCtx {
@@ -110,22 +92,31 @@ __device__ __forceinline__ Origin origin_of(const MoveCtx<Real>& m, uint32_t gc)
 // same cell in a channel of two rows) gets o bin + k, with o = (3 (dz + 1) + dy + 1) 3 + dx + 1
 // (dz = 0 in 2D, o < 9) and k its rank in its old cell; any other particle bit 31 and its
 // origin slot, old cell bin + k, so it follows the near ones. Keys are distinct within a cell.
+constexpr uint32_t kFarOffset = 0xFFu;
 template <typename Real, bool Z3>
-__device__ __forceinline__ uint32_t order_key(const MoveCtx<Real>& m, const Origin& o, uint32_t k, int ix,
-                                              int iy, int iz) {
-    const int dx = ix - o.x;
-    int ey = iy - o.y;
-    if (ey < 0) ey += m.ncy;
-    const int dy = ey == 0 ? 0 : (ey == 1 ? 1 : (ey == m.ncy - 1 ? -1 : 2));
-    int dz = 0;
+__device__ __forceinline__ uint32_t neighbour_offset(const MoveCtx<Real>& m, const Origin& o, int ix, int iy,
+                                                     int iz) {
+    // displacements plus one along each axis, 0 to 2 for a neighbour
+    const uint32_t ux = (uint32_t)(ix - o.x + 1);
+    auto wrapped = [](int d, int period) -> uint32_t {
+        int u = d + 1;
+        if (u < (period == 2 ? 1 : 0)) u += period;  // (a period of two: -1 is +1)
+        if (u > 2) u -= period;
+        return (uint32_t)u;
+    };
+    const uint32_t uy = wrapped(iy - o.y, m.ncy);
+    uint32_t off = 3u * uy + ux;
+    bool far = ux > 2u || uy > 2u;
     if constexpr (Z3) {
-        int ez = iz - o.z;
-        if (ez < 0) ez += m.ncz;
-        dz = ez == 0 ? 0 : (ez == 1 ? 1 : (ez == m.ncz - 1 ? -1 : 2));
+        const uint32_t uz = wrapped(iz - o.z, m.ncz);
+        off += 9u * uz;
+        far = far || uz > 2u;
     }
-    if (dx < -1 || dx > 1 || dy > 1 || dz > 1) return 0x80000000u | (o.gc * m.bin + k);
-    const int off = (Z3 ? 9 * (dz + 1) : 0) + 3 * (dy + 1) + (dx + 1);
-    return (uint32_t)off * m.bin + k;
+    return far ? kFarOffset : off;
+}
+template <typename Real>
+__device__ __forceinline__ uint32_t order_key(const MoveCtx<Real>& m, const Origin& o, uint32_t k, uint32_t off) {
+    return off == kFarOffset ? 0x80000000u | (o.gc * m.bin + k) : off * m.bin + k;
 }
 
 // Diffuse isothermal re-emission from a wall at rest: normal speed sqrt(-2 ln U) into the
@@ -189,18 +180,12 @@ __device__ __forceinline__ Real wrap_periodic(Real v, Real period) {
 }
 
 // Kick (v_y += g), then the flight of one step from (px, py, pz) with walls and periodic
-// wrap; the particle is rank k of the channel's cell o at the start of step s (the key of its
-// wall draws). Returns its new cell of the context, (iz nly + iy - y0) ncx + ix, with dir = -1;
-// for a particle that leaves a streamwise slab, the channel's cell (iz ncy + iy) ncx + ix and
-// dir = 0 (towards lower rows) or 1 (higher rows, across the periodic end included). `key` is
-// its order key in the new cell. SLAB = false: the context holds the whole channel (y0 = 0,
-// nly = ncy), which no particle leaves.
-template <typename Real, bool Z3, bool SLAB = true>
-__device__ __forceinline__ uint32_t move_particle(const MoveCtx<Real>& m, const Origin& o, uint32_t k,
-                                                  uint32_t s, Real& px, Real& py, Real& pz, Real& ux,
-                                                  Real& uy, Real& uz, uint32_t& hits, uint32_t& caps,
-                                                  int& dir, uint32_t& key) {
-    const uint32_t c = o.gc;
+// wrap, of the particle of rank k of the channel's cell o at the start of step s (the key of its
+// wall draws); its new column, channel row and layer.
+template <typename Real, bool Z3>
+__device__ __forceinline__ void fly(const MoveCtx<Real>& m, const Origin& o, uint32_t k, uint32_t s, Real& px,
+                                    Real& py, Real& pz, Real& ux, Real& uy, Real& uz, uint32_t& hits,
+                                    uint32_t& caps, int& ix, int& iy, int& iz) {
     uy = uy + m.g;
     const Real xn = px + ux * m.dt;
     if (xn >= (Real)0 && xn <= m.H) {
@@ -208,23 +193,32 @@ __device__ __forceinline__ uint32_t move_particle(const MoveCtx<Real>& m, const 
         py = py + uy * m.dt;
         if constexpr (Z3) pz = pz + uz * m.dt;
     } else {
-        wall_flight<Real, Z3>(m.seed, c, k, s, m.H, m.dt, px, py, ux, uy, uz, hits, caps, pz);
+        wall_flight<Real, Z3>(m.seed, o.gc, k, s, m.H, m.dt, px, py, ux, uy, uz, hits, caps, pz);
     }
     py = wrap_periodic(py, m.L);
-    int ix = (int)floor(px), iy = (int)floor(py);
+    ix = (int)floor(px), iy = (int)floor(py);
     ix = ix < 0 ? 0 : (ix > m.ncx - 1 ? m.ncx - 1 : ix);
     iy = iy < 0 ? 0 : (iy > m.ncy - 1 ? m.ncy - 1 : iy);
-    int iz = 0;
+    iz = 0;
     if constexpr (Z3) {
         pz = wrap_periodic(pz, m.Lz);
         iz = (int)floor(pz);
         iz = iz < 0 ? 0 : (iz > m.ncz - 1 ? m.ncz - 1 : iz);
     }
-    key = order_key<Real, Z3>(m, o, k, ix, iy, iz);
-    if constexpr (!SLAB) {
-        dir = -1;
-        return (uint32_t)((iz * m.ncy + iy) * m.ncx + ix);
-    }
+}
+
+// The move of one particle (fly). Returns its new cell of the context, (iz nly + iy - y0) ncx + ix,
+// with dir = -1; for a particle that leaves a streamwise slab, the channel's cell
+// (iz ncy + iy) ncx + ix and dir = 0 (towards lower rows) or 1 (higher rows, across the periodic
+// end included). `key` is its order key in the new cell.
+template <typename Real, bool Z3>
+__device__ __forceinline__ uint32_t move_particle(const MoveCtx<Real>& m, const Origin& o, uint32_t k,
+                                                  uint32_t s, Real& px, Real& py, Real& pz, Real& ux,
+                                                  Real& uy, Real& uz, uint32_t& hits, uint32_t& caps,
+                                                  int& dir, uint32_t& key) {
+    int ix, iy, iz;
+    fly<Real, Z3>(m, o, k, s, px, py, pz, ux, uy, uz, hits, caps, ix, iy, iz);
+    key = order_key(m, o, k, neighbour_offset<Real, Z3>(m, o, ix, iy, iz));
     const int iyl = iy - m.y0;
     if (iyl >= 0 && iyl < m.nly) {
         dir = -1;

@@ -274,6 +274,12 @@ __device__ __forceinline__ void cp_async16(void* smem, const void* gmem) {
     const unsigned s = (unsigned)__cvta_generic_to_shared(smem);
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(s), "l"(gmem) : "memory");
 }
+// The same for 4, 8 or 16 bytes through L1 (copies of the parts of one sector share its fetch).
+template <int BYTES>
+__device__ __forceinline__ void cp_async_part(void* smem, const void* gmem) {
+    const unsigned s = (unsigned)__cvta_generic_to_shared(smem);
+    asm volatile("cp.async.ca.shared.global [%0], [%1], %2;" ::"r"(s), "l"(gmem), "n"(BYTES) : "memory");
+}
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
 __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 
@@ -633,7 +639,7 @@ struct Ctx {
     bool split_pending = false;    // a slab's dsmc_move was issued, its collide is due
     int fuse_mode = 0;             // HYB_FUSE_*: multi-step calls fuse the DSMC passes
     int fuse_pays = -1;            // HYB_FUSE_AUTO's choice, formed at the first multi-step call
-    int collide_warps = 8;         // collide block shape: 8 warps (32 cells) or 4 (16 cells)
+    int collide_warps = 4;         // collide block shape: 8 warps (32 cells) or 4 (16 cells)
     // hyb_hybrid_step_host: device staging of the lists and the gathered moment sums, and a
     // ring of completion events of the steps in flight
     char* io_dev = nullptr;

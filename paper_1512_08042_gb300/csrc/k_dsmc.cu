@@ -102,20 +102,6 @@ __global__ void k_init_cells(DsmcArgs<Real> a) {
     }
 }
 
-// Exact widening of a float to double on the integer pipe (the FP64 pipe is slow on this
-// part): a normal float's sign, exponent rebiased from 127 to 1023 and mantissa shifted to
-// the top of the 52-bit field (IEEE 754 binary32 and binary64 formats). Zeros, subnormals,
-// infinities and NaNs take the plain conversion.
-__device__ __forceinline__ double widen(float f) {
-    const uint32_t u = __float_as_uint(f);
-    const uint32_t e = (u >> 23) & 0xFFu;
-    if (e == 0u || e == 0xFFu) return (double)f;
-    const uint64_t bits = ((uint64_t)(u >> 31) << 63) | ((uint64_t)(e + 896u) << 52) |
-                          ((uint64_t)(u & 0x7FFFFFu) << 29);
-    return __longlong_as_double((long long)bits);
-}
-__device__ __forceinline__ double widen(double d) { return d; }
-
 // ---------------------------------------------------------------------------------------
 // Move (kick, drift, walls, wrap) of the sorted particles of half p into the bins of p^1.
 
@@ -231,16 +217,21 @@ __global__ void __launch_bounds__(256, 4) k_move(Launch<DsmcArgs<Real>> L) {
 // every shuffle is executed by the full warp.
 //
 // Bound by latency and issue, not by bandwidth (ncu, 6.55M particles with Kn along the channel:
-// issue 48%, DRAM 30% of its peak, 16.7 warp instructions per particle). No block barrier: while
-// one warp of a block ran the block's NTC chains and the others waited, barriers were a fifth of
-// the stalls. 20 steps, before and after: 105M particles 78.0 -> 70.3 ms, 819k 2.17 -> 1.50 ms,
-// 3D 6.55M 13.6 -> 9.6 ms, 64 batched channels (10 steps) 1.50 -> 1.19 ms.
+// issue 52%, DRAM a third of its peak, 15.9 warp instructions per particle). No block barrier:
+// while one warp of a block ran the block's NTC chains and the others waited, barriers were a
+// fifth of the stalls (105M particles, 20 steps: 78.0 ms; warps on their own: 70.3 ms). The
+// arrivals are copied to shared memory by asynchronous copies and stay where they land, a byte
+// per rank pointing at them, and a cell's particles bound for one neighbour share one
+// reservation of slots there, all nine in flight together, instead of one dependent global
+// atomic per eight particles (61.7 ms; 819k particles 2.17 -> 1.35 ms, 3D 6.55M
+// 13.6 -> 9.0 ms, 64 batched channels, 10 steps, 1.50 -> 1.04 ms).
 constexpr int kGroup = 8;
 constexpr int kWarpCells = 32 / kGroup;
 
-// Blocks of 8 warps (32 cells) or 4 (16 cells) only group warps for a launch. 24 resident warps
-// per SM in FP32 (80 registers): 20, 28 and 32 warps took 72.6, 75.0 and 90.8 ms for the 105M
-// particles' 20 steps against 70.8 ms, more warps spilling what the held arrivals need.
+// Blocks of 8 warps (32 cells) or 4 (16 cells) only group warps for a launch: a block keeps its
+// shared memory until its slowest warp is done, so 4 are faster where the grid runs many waves
+// (105M particles, 20 steps: 61.7 against 63.7 ms) and 8 by 2% where it does not. 24 resident warps
+// per SM in FP32 (80 registers): 28 took 67.2 ms (spills, and little L1 left beside the pools).
 constexpr int kCollideWarps = 8;
 template <typename Real, int W>
 struct CollideCfg {
@@ -248,30 +239,54 @@ struct CollideCfg {
 };
 enum CollideMode : int { MODE_COLLIDE = 0, MODE_FUSED = 1 };
 
-// Real arrays of the shared-memory pool per slot: vx, vy, vz, x, y (, z)
-template <bool Z3>
-__host__ __device__ constexpr int pool_reals() {
-    return Z3 ? 6 : 5;
-}
-
 // Words of a cell's order-key bitmap: one bit per key below W bin, W = 9 neighbour offsets in
 // 2D and 27 in 3D (bin is a multiple of 32).
 template <bool Z3>
+__host__ __device__ constexpr int neighbours() {
+    return Z3 ? 27 : 9;
+}
+template <bool Z3>
 __host__ __device__ constexpr int bitmap_words(uint32_t bin) {
-    return (Z3 ? 27 : 9) * (int)(bin / 32u);
+    return neighbours<Z3>() * (int)(bin / 32u);
 }
 // Keys of farther-displaced particles a cell lists for their ranks (more are counted in full).
 constexpr int kFarList = 8;
 
-// Shared memory of one warp: the pool of its cells' particles (pool_reals Real per slot), then
-// its cells' key bitmaps (words, listed far keys, prefix bytes), in whose place the cells'
-// FP64 sums are copied in once the ranks are taken.
+// Shared memory of one warp, byte offsets: per slot of its pool (x, y, vx, vy), then vz (, z), the
+// order key (after the collide: the slot's place in its new cell) and the slot of each rank; then
+// the cells' key bitmaps (words, listed far keys, prefix bytes), in whose place come, once the
+// ranks are taken, the cells' FP64 sums and the slots reserved in each neighbour's bin.
+struct WarpMem {
+    uint32_t b, key, perm, scratch, total;
+};
 template <typename Real, bool Z3>
-__host__ __device__ constexpr uint32_t collide_warp_smem(uint32_t pool, uint32_t bin) {
+__host__ __device__ constexpr WarpMem warp_mem(uint32_t pool, uint32_t bin) {
+    WarpMem m{};
+    m.b = pool * 4u * (uint32_t)sizeof(Real);  // pool is a multiple of 8
+    m.key = m.b + pool * (Z3 ? 2u : 1u) * (uint32_t)sizeof(Real);
+    m.perm = m.key + pool * 4u;
+    m.scratch = (m.perm + pool + 15u) / 16u * 16u;
     const uint32_t bits = (uint32_t)kWarpCells * ((uint32_t)bitmap_words<Z3>(bin) * 5u + (kFarList + 1u) * 4u);
-    const uint32_t sums = (uint32_t)kWarpCells * kMoments * 8u;
-    const uint32_t pv = (pool * (uint32_t)(pool_reals<Z3>() * sizeof(Real)) + 15u) / 16u * 16u;
-    return pv + ((bits > sums ? bits : sums) + 15u) / 16u * 16u;
+    const uint32_t after = (uint32_t)kWarpCells * (kMoments * 8u + (uint32_t)neighbours<Z3>() * 8u);
+    m.total = m.scratch + ((bits > after ? bits : after) + 15u) / 16u * 16u;
+    return m;
+}
+
+// Four Reals of shared memory, 16-byte aligned (32 in FP64), as vector accesses.
+__device__ __forceinline__ void get4(const float* p, float& a, float& b, float& c, float& d) {
+    const float4 v = *reinterpret_cast<const float4*>(p);
+    a = v.x, b = v.y, c = v.z, d = v.w;
+}
+__device__ __forceinline__ void get4(const double* p, double& a, double& b, double& c, double& d) {
+    const double2 u = *reinterpret_cast<const double2*>(p), v = *reinterpret_cast<const double2*>(p + 2);
+    a = u.x, b = u.y, c = v.x, d = v.y;
+}
+__device__ __forceinline__ void put4(float* p, float a, float b, float c, float d) {
+    *reinterpret_cast<float4*>(p) = make_float4(a, b, c, d);
+}
+__device__ __forceinline__ void put4(double* p, double a, double b, double c, double d) {
+    *reinterpret_cast<double2*>(p) = make_double2(a, b);
+    *reinterpret_cast<double2*>(p + 2) = make_double2(c, d);
 }
 
 // Adds a particle's velocity moments to a lane's partial sums: u, the six distinct products
@@ -291,45 +306,61 @@ __device__ __forceinline__ void add_moments(Real (&mo)[kMoments], Real ux, Real 
     mo[18] = fma(zz, uy, mo[18]); mo[19] = fma(zz, uz, mo[19]);
 }
 
-// The NTC candidates of a cell group's cell (nsel of them, n particles, velocities at vx, vy,
-// vz), applied in their order. The cell's lanes draw eight consecutive candidates at a time and
-// settle them together: every pending lane forms its relative speed from the current
-// velocities, the running (sigma c_r)_max up to its candidate by a prefix maximum and its
-// decision; a candidate that shares a particle with an earlier one of the window that collides
-// must see that collision, so the candidates before the first such one are final and the others
-// are taken again from the updated velocities. The results are those of applying the candidates
-// one after another, bit for bit. Shared particles are found with 64-bit sets of the particles
-// (index modulo 64; an alias only takes a candidate again). The first pending candidate is
-// always final, so every pass settles at least one.
+// One NTC candidate: the pair (ranks in the cell), the acceptance uniform and the direction of
+// the relative velocity after the collision (ok = 0 if its draws ran out).
 template <typename Real>
-__device__ __forceinline__ void ntc_collisions(uint64_t seed, uint32_t gc, uint32_t s, uint32_t n, uint32_t nsel,
-                                               Real* vx, Real* vy, Real* vz, int grp, int gl, Real& cm,
-                                               uint32_t& ncoll, uint32_t& flags) {
+struct Candidate {
+    uint32_t i, j;
+    Real R, nx, ny, nz;
+    int ok;
+};
+template <typename Real>
+__device__ __forceinline__ void draw_candidate(Candidate<Real>& q, uint64_t seed, uint32_t gc, uint32_t s,
+                                               uint32_t n, uint32_t k) {
+    const uint4 r = draw(seed, gc, s, TAG_NTC_PAIR, k, 0);
+    q.i = uindex(r.x, n);
+    q.j = uindex(r.y, n - 1u);
+    if (q.j >= q.i) q.j += 1u;
+    q.R = (Real)u01f(r.z);
+    q.ok = unit_vector(seed, gc, s, k, q.nx, q.ny, q.nz);
+}
+
+// The NTC candidates of a cell group's cell (nsel of them, n particles; `va` and `vb` point at
+// (vx, vy) and vz of slot 0, 4 and NB Reals a slot, perm gives the slot of each rank), applied in
+// their order; q holds the lane's candidate of the first eight. The cell's lanes take eight
+// consecutive candidates at a time and settle them together: every pending lane forms its
+// relative speed from the current velocities, the running (sigma c_r)_max up to its candidate by
+// a prefix maximum and its decision; a candidate that shares a particle with an earlier one of
+// the window that collides must see that collision, so the candidates before the first such one
+// are final and the others are taken again from the updated velocities. The results are those of
+// applying the candidates one after another, bit for bit. Shared particles are found with 64-bit
+// sets of the particles (index modulo 64; an alias only takes a candidate again). The first
+// pending candidate is always final, so every pass settles at least one.
+template <typename Real, int NB>
+__device__ __forceinline__ void ntc_collisions(Candidate<Real>& q, uint64_t seed, uint32_t gc, uint32_t s, uint32_t n,
+                                               uint32_t nsel, Real* va, Real* vb, const uint8_t* perm, int grp,
+                                               int gl, Real& cm, uint32_t& ncoll, uint32_t& flags) {
     constexpr int G = kGroup;
     const uint32_t maxsel = __reduce_max_sync(kFull, nsel);
     for (uint32_t k0 = 0; k0 < maxsel; k0 += G) {
         const uint32_t k = k0 + (uint32_t)gl;
         bool pend = k < nsel;
-        uint32_t i = 0, j = 0;
-        Real R = (Real)0, nx = (Real)0, ny = (Real)0, nz = (Real)0;
-        int ok = 0;
-        if (pend) {
-            const uint4 r = draw(seed, gc, s, TAG_NTC_PAIR, k, 0);
-            i = uindex(r.x, n);
-            j = uindex(r.y, n - 1u);
-            if (j >= i) j += 1u;
-            R = (Real)u01f(r.z);
-            ok = unit_vector(seed, gc, s, k, nx, ny, nz);
-        }
-        const uint32_t bi = 1u << (i & 31u), bj = 1u << (j & 31u);
-        const uint32_t mlo = ((i & 32u) ? 0u : bi) | ((j & 32u) ? 0u : bj);
-        const uint32_t mhi = ((i & 32u) ? bi : 0u) | ((j & 32u) ? bj : 0u);
+        if (k0 > 0 && pend) draw_candidate(q, seed, gc, s, n, k);
+        uint32_t pi = 0, pj = 0;
+        if (pend) pi = perm[q.i], pj = perm[q.j];
+        Real* ai = va + 4 * pi;
+        Real* aj = va + 4 * pj;
+        Real* bi = vb + NB * pi;
+        Real* bj = vb + NB * pj;
+        const uint32_t si = 1u << (q.i & 31u), sj = 1u << (q.j & 31u);
+        const uint32_t mlo = ((q.i & 32u) ? 0u : si) | ((q.j & 32u) ? 0u : sj);
+        const uint32_t mhi = ((q.i & 32u) ? si : 0u) | ((q.j & 32u) ? sj : 0u);
         while (__any_sync(kFull, pend)) {
             Real ax = 0, ay = 0, az = 0, bx = 0, by = 0, bz = 0, cr = 0;
             Real v = cm;
             if (pend) {
-                ax = vx[i], ay = vy[i], az = vz[i];
-                bx = vx[j], by = vy[j], bz = vz[j];
+                ax = ai[0], ay = ai[1], az = bi[0];
+                bx = aj[0], by = aj[1], bz = bj[0];
                 const Real ddx = ax - bx, ddy = ay - by, ddz = az - bz;
                 cr = sqrt(ddx * ddx + ddy * ddy + ddz * ddz);
                 if (cr > cm) v = cr;
@@ -339,8 +370,8 @@ __device__ __forceinline__ void ntc_collisions(uint64_t seed, uint32_t gc, uint3
                 const Real t = __shfl_up_sync(kFull, v, o, G);
                 if (gl >= o && t > v) v = t;
             }
-            const bool acc = pend && cr > R * v;
-            const bool coll = acc && ok;
+            const bool acc = pend && cr > q.R * v;
+            const bool coll = acc && q.ok;
             uint32_t elo = coll ? mlo : 0u, ehi = coll ? mhi : 0u;
 #pragma unroll
             for (int o = 1; o < G; o <<= 1) {
@@ -360,13 +391,13 @@ __device__ __forceinline__ void ntc_collisions(uint64_t seed, uint32_t gc, uint3
                     const Real cy = (ay + by) * (Real)0.5;
                     const Real cz = (az + bz) * (Real)0.5;
                     const Real h = cr * (Real)0.5;
-                    const Real hx = h * nx, hy = h * ny, hz = h * nz;
-                    vx[i] = cx + hx;
-                    vy[i] = cy + hy;
-                    vz[i] = cz + hz;
-                    vx[j] = cx - hx;
-                    vy[j] = cy - hy;
-                    vz[j] = cz - hz;
+                    const Real hx = h * q.nx, hy = h * q.ny, hz = h * q.nz;
+                    ai[0] = cx + hx;
+                    ai[1] = cy + hy;
+                    bi[0] = cz + hz;
+                    aj[0] = cx - hx;
+                    aj[1] = cy - hy;
+                    bj[0] = cz - hz;
                     ncoll += 1;
                 } else if (acc) {
                     flags |= HYB_ST_SCATTER_CAP;
@@ -388,28 +419,26 @@ __device__ __forceinline__ void collide_warp(const DsmcArgs<Real>& a, uint32_t p
                                              uint32_t& ncand, uint32_t& ncoll, uint32_t& nlive,
                                              uint32_t& flags) {
     constexpr int G = kGroup;
-    constexpr int NR = pool_reals<Z3>();
-    // FP32: the first SMALL arrivals of a cell are held in registers between the marking of
-    // their keys and their placement (48 or 32 held: 72.2 or 77.4 ms against 70.8 ms, none 80.3 ms,
-    // at 105M particles); FP64 (twice the registers) reads them again
-    constexpr int SMALL = 64;
-    constexpr int R = SMALL / G;
-    constexpr bool HELD = sizeof(Real) == 4;
-    constexpr int SJ = 2;  // arrivals per lane whose loads are in flight together when read again
+    constexpr int NB = Z3 ? 2 : 1;
+    constexpr int NOFF = neighbours<Z3>();
+    constexpr int RB = (int)sizeof(Real);
     const unsigned lane = lane_id();
     const int grp = (int)lane / G, gl = (int)lane % G;
     const uint32_t bin = (uint32_t)a.bin;
-    Real* pv = reinterpret_cast<Real*>(smem);
-    unsigned char* scratch = smem + ((size_t)pool * NR * sizeof(Real) + 15) / 16 * 16;
+    const WarpMem wm = warp_mem<Real, Z3>(pool, bin);
+    unsigned char* scratch = smem + wm.scratch;
     const int BW = bitmap_words<Z3>(bin);
     const int CW = (BW + G - 1) / G;
     const uint32_t lim = (uint32_t)BW * 32u;
     uint32_t* bm = reinterpret_cast<uint32_t*>(scratch) + grp * BW;
     uint32_t* fl = reinterpret_cast<uint32_t*>(scratch) + kWarpCells * BW + grp * (kFarList + 1);
     uint8_t* pf = scratch + (size_t)kWarpCells * (BW + kFarList + 1) * 4 + grp * BW;
-    double* sums = reinterpret_cast<double*>(scratch) + grp * kMoments;  // after the ranks
+    // after the ranks: the cell's sums, and per neighbour the particles bound for it, then the
+    // first of their slots and how many of them fit
+    double* sums = reinterpret_cast<double*>(scratch) + grp * kMoments;
+    uint2* dest = reinterpret_cast<uint2*>(scratch + kWarpCells * kMoments * 8) + grp * NOFF;
     const uint32_t s = a.ctrl[CTRL_STEP];
-    const bool do_sample = (s % (uint32_t)a.sample_every) == 0u;
+    const bool do_sample = a.sample_every == 1 || (s % (uint32_t)a.sample_every) == 0u;
     uint32_t hits = 0, caps = 0, lost = 0;
 
     const int c = cell0 + grp;
@@ -419,13 +448,6 @@ __device__ __forceinline__ void collide_warp(const DsmcArgs<Real>& a, uint32_t p
     const uint32_t gc = global_cell((uint32_t)c, a.ncx, a.ncy, a.y0, a.ncy_g);
     const Real* __restrict__ drec = a.drec;
     uint32_t n_all = has ? a.count_d[c] : 0u;
-    // the first half of the held arrivals is read beside the count (a bin has at least 32 slots)
-    Held<Real, R> held;
-    if constexpr (HELD) {
-#pragma unroll
-        for (int r = 0; r < R / 2; ++r)
-            if (has) held.load(drec, base + gl + G * r, r);
-    }
     uint32_t nb0 = 0;
     Real cm0 = (Real)0, rem0 = (Real)0;
     if (has) {
@@ -435,11 +457,6 @@ __device__ __forceinline__ void collide_warp(const DsmcArgs<Real>& a, uint32_t p
     }
     const bool moving = MODE == MODE_FUSED && has && !(a.coupled && a.coupled[c]);
     if (n_all > bin) n_all = bin;
-    if constexpr (HELD) {
-#pragma unroll
-        for (int r = R / 2; r < R; ++r)
-            if ((uint32_t)(gl + G * r) < n_all) held.load(drec, base + gl + G * r, r);
-    }
     // the cells' regions of the warp's pool (exclusive sums of the counts); if they do not
     // fit, the cells take the whole pool one after another
     uint32_t off = 0, tot = 0;
@@ -450,134 +467,37 @@ __device__ __forceinline__ void collide_warp(const DsmcArgs<Real>& a, uint32_t p
         tot += t;
     }
     const bool fits = tot <= pool;
+    if (!fits) off = 0;
     const int rounds = fits ? 1 : kWarpCells;
+    Real* va = reinterpret_cast<Real*>(smem) + 4 * off;
+    Real* vb = reinterpret_cast<Real*>(smem + wm.b) + NB * off;
+    uint32_t* key = reinterpret_cast<uint32_t*>(smem + wm.key) + off;
+    uint8_t* perm = smem + wm.perm + off;
 
-    // A. stable order: every arrival's rank among the cell's arrivals by order key. A key
-    // below W bin (a particle from a neighbouring cell) sets bit `key` of the cell's
-    // bitmap, and its rank is the number of set bits below it: the count before its word
-    // (a prefix over the words, kept modulo 256: a queried word holds its own bit, so
-    // the count is below bin) plus those below it within the word. Larger keys follow
-    // all of these, each ranked by counting the larger keys below it (from a list of the
-    // cell's larger keys while they are few, else from the records).
-    auto clear_keys = [&]() {
-        for (int q = gl; q < BW; q += G) bm[q] = 0u;
-        if (gl == 0) fl[0] = 0u;
-        __syncwarp();
-    };
-    auto mark_key = [&](uint32_t t) {
-        if (t < lim) {
-            atomicOr(&bm[t >> 5], 1u << (t & 31u));
-        } else {
-            const uint32_t j = atomicAdd(&fl[0], 1u);
-            if (j < (uint32_t)kFarList) fl[1 + j] = t;
-        }
-    };
-    auto count_keys = [&]() {  // the prefix counts: lane gl owns words [gl CW, gl CW + CW)
-        __syncwarp();
-        const int q0 = gl * CW, q1 = min(q0 + CW, BW);
-        uint32_t mine = 0;
-        for (int q = q0; q < q1; ++q) mine += (uint32_t)__popc(bm[q]);
-        uint32_t inc = mine;
-#pragma unroll
-        for (int o = 1; o < G; o <<= 1) {
-            const uint32_t t = __shfl_up_sync(kFull, inc, o, G);
-            if (gl >= o) inc += t;
-        }
-        uint32_t run = inc - mine;
-        for (int q = q0; q < q1; ++q) {
-            pf[q] = (uint8_t)run;
-            run += (uint32_t)__popc(bm[q]);
-        }
-        __syncwarp();
-    };
-    auto rank_of = [&](uint32_t t, uint32_t n) -> uint32_t {
-        if (t < lim) {
-            const uint32_t q = t >> 5;
-            return (uint32_t)pf[q] + (uint32_t)__popc(bm[q] & ((1u << (t & 31u)) - 1u));
-        }
-        const uint32_t nfar = fl[0];
-        uint32_t rk = n - nfar;
-        if (nfar <= (uint32_t)kFarList) {
-            for (uint32_t m2 = 0; m2 < nfar; ++m2) rk += fl[1 + m2] < t ? 1u : 0u;
-        } else {
-            for (uint32_t m2 = 0; m2 < n; ++m2) {
-                const uint32_t u = rec_tag(drec, base + m2);
-                rk += (u >= lim && u < t) ? 1u : 0u;
-            }
-        }
-        return rk;
-    };
-    auto place = [&](Real* v, uint32_t rk, Real px, Real py, Real pz, Real ux, Real uy, Real uz) {
-        v[rk] = ux;
-        v[pool + rk] = uy;
-        v[2 * pool + rk] = uz;
-        v[3 * pool + rk] = px;
-        v[4 * pool + rk] = py;
-        if constexpr (Z3) v[5 * (size_t)pool + rk] = pz;
-    };
-    // the arrivals from slot k_first on, read (again) from the records
-    auto place_from = [&](Real* v, uint32_t k_first, uint32_t n) {
-        for (uint32_t k0 = k_first; k0 < n; k0 += SJ * G) {
-            Real p[SJ][6];
-            uint32_t t[SJ];
-#pragma unroll
-            for (int j = 0; j < SJ; ++j) {
-                const uint32_t k = k0 + (uint32_t)(gl + G * j);
-                if (k < n) rec_get(drec, base + k, p[j][0], p[j][1], p[j][2], p[j][3], p[j][4], p[j][5], t[j]);
-            }
-#pragma unroll
-            for (int j = 0; j < SJ; ++j) {
-                const uint32_t k = k0 + (uint32_t)(gl + G * j);
-                if (k < n) place(v, rank_of(t[j], n), p[j][0], p[j][1], p[j][2], p[j][3], p[j][4], p[j][5]);
-            }
-        }
-    };
-    constexpr uint32_t K0 = HELD ? (uint32_t)SMALL : 0u;  // arrivals from here on are not held
-    if (fits) {
-        clear_keys();
-        if constexpr (HELD) {
-#pragma unroll
-            for (int r = 0; r < R; ++r)
-                if ((uint32_t)(gl + G * r) < n_all) mark_key(held.key(r));
-        }
-        for (uint32_t k = K0 + gl; k < n_all; k += G) mark_key(rec_tag(drec, base + k));
-        count_keys();
-        if constexpr (HELD) {
-#pragma unroll
-            for (int r = 0; r < R; ++r)
-                if ((uint32_t)(gl + G * r) < n_all) {
-                    Real p[6];
-                    held.get(r, p);
-                    place(pv + off, rank_of(held.key(r), n_all), p[0], p[1], p[2], p[3], p[4], p[5]);
-                }
-        }
-        place_from(pv + off, K0, n_all);
-        __syncwarp();
-    }
     for (int round = 0; round < rounds; ++round) {
         const bool act = fits || grp == round;
         const bool has_r = has && act;
         const uint32_t n = act ? n_all : 0u;
-        Real* vx = pv + (fits ? off : 0u);
-        Real* vy = vx + pool;
-        Real* vz = vx + 2 * pool;
-        Real* qx = vx + 3 * pool;
-        Real* qy = vx + 4 * pool;
-        Real* qz = vx + 5 * (size_t)pool;  // 3D only
-        if (!fits) {
-            clear_keys();
-            for (uint32_t k = gl; k < n; k += G) mark_key(rec_tag(drec, base + k));
-            count_keys();
-            place_from(vx, 0u, n);
-            __syncwarp();
+        // every loop over a cell's particles runs as often as the fullest cell of the warp needs,
+        // its lanes masked: trip counts of their own would have the warp run a loop's unrolled
+        // body and its remainder one after the other
+        const uint32_t nmax = __reduce_max_sync(kFull, n);
+        // the cell's arrivals, copied to shared memory (no registers hold them, so all of a
+        // warp's loads are in flight together)
+#pragma unroll 2
+        for (uint32_t k0 = 0; k0 < nmax; k0 += G) {
+            const uint32_t k = k0 + (uint32_t)gl;
+            if (k < n) {
+                const Real* r = drec + (base + k) * kRec;
+                cp_async_part<16>(va + 4 * k, r);
+                if constexpr (RB == 8) cp_async_part<16>(va + 4 * k + 2, r + 2);
+                cp_async_part<NB * RB>(vb + NB * k, r + RS_VZ);
+                cp_async_part<4>(key + k, r + RS_TAG);
+            }
         }
-        // the ranks are taken: the cell's FP64 sums are copied over the bitmaps while the cell
-        // is collided (10 x 16 bytes)
-        if (has_r && do_sample)
-            for (int j = gl; j < kMoments / 2; j += G)
-                cp_async16(&sums[2 * j], &a.acc[(size_t)c * kMoments + 2 * j]);
         cp_async_commit();
-        // B. N_cand = 1/2 N Nbar F_N (sigma c_r)_max dt / V_c + remainder, and the candidates
+        // N_cand = 1/2 N Nbar F_N (sigma c_r)_max dt / V_c + remainder, and the first eight
+        // candidates, while the arrivals come in
         uint32_t nsel = 0;
         Real cm = cm0;
         if (has_r) {
@@ -601,8 +521,90 @@ __device__ __forceinline__ void collide_warp(const DsmcArgs<Real>& a, uint32_t p
                 ncand += nsel;
             }
         }
-        ntc_collisions(a.seed, gc, s, n, nsel, vx, vy, vz, grp, gl, cm, ncoll, flags);
+        Candidate<Real> cand{};
+        if ((uint32_t)gl < nsel) draw_candidate(cand, a.seed, gc, s, n, (uint32_t)gl);
+        // A. stable order: every arrival's rank among the cell's arrivals by order key. A key
+        // below W bin (a particle from a neighbouring cell) sets bit `key` of the cell's
+        // bitmap, and its rank is the number of set bits below it: the count before its word
+        // (a prefix over the words, kept modulo 256: a queried word holds its own bit, so
+        // the count is below bin) plus those below it within the word. Larger keys follow
+        // all of these, each ranked by counting the larger keys below it (from a list of the
+        // cell's larger keys while they are few, else from all keys).
+        for (int q0 = 0; q0 < BW; q0 += G)
+            if (q0 + gl < BW) bm[q0 + gl] = 0u;
+        if (gl == 0) fl[0] = 0u;
+        cp_async_wait_all();
+        __syncwarp();
+#pragma unroll 2
+        for (uint32_t k0 = 0; k0 < nmax; k0 += G) {
+            const uint32_t k = k0 + (uint32_t)gl;
+            if (k >= n) continue;
+            const uint32_t t = key[k];
+            if (t < lim) {
+                atomicOr(&bm[t >> 5], 1u << (t & 31u));
+            } else {
+                const uint32_t j = atomicAdd(&fl[0], 1u);
+                if (j < (uint32_t)kFarList) fl[1 + j] = t;
+            }
+        }
+        __syncwarp();
+        {  // the prefix counts: lane gl owns words [gl CW, gl CW + CW)
+            const int q0 = gl * CW;
+            uint32_t mine = 0;
+            for (int i = 0; i < CW; ++i)
+                if (q0 + i < BW) mine += (uint32_t)__popc(bm[q0 + i]);
+            uint32_t inc = mine;
+#pragma unroll
+            for (int o = 1; o < G; o <<= 1) {
+                const uint32_t t = __shfl_up_sync(kFull, inc, o, G);
+                if (gl >= o) inc += t;
+            }
+            uint32_t run = inc - mine;
+            for (int i = 0; i < CW; ++i)
+                if (q0 + i < BW) {
+                    pf[q0 + i] = (uint8_t)run;
+                    run += (uint32_t)__popc(bm[q0 + i]);
+                }
+        }
+        __syncwarp();
+#pragma unroll 2
+        for (uint32_t k0 = 0; k0 < nmax; k0 += G) {
+            const uint32_t k = k0 + (uint32_t)gl;
+            if (k >= n) continue;
+            const uint32_t t = key[k];
+            uint32_t rk;
+            if (t < lim) {
+                const uint32_t q = t >> 5;
+                rk = (uint32_t)pf[q] + (uint32_t)__popc(bm[q] & ((1u << (t & 31u)) - 1u));
+            } else {
+                const uint32_t nfar = fl[0];
+                rk = n - nfar;
+                if (nfar <= (uint32_t)kFarList) {
+                    for (uint32_t m2 = 0; m2 < nfar; ++m2) rk += fl[1 + m2] < t ? 1u : 0u;
+                } else {
+                    for (uint32_t m2 = 0; m2 < n; ++m2) rk += (key[m2] >= lim && key[m2] < t) ? 1u : 0u;
+                }
+            }
+            perm[rk] = (uint8_t)k;
+        }
+        __syncwarp();
+        // the ranks are taken: the cell's FP64 sums are copied over the bitmaps while the cell
+        // is collided (10 x 16 bytes), and the neighbours' counts start at zero
+        if (has_r && do_sample)
+#pragma unroll
+            for (int i = 0; i < (kMoments / 2 + G - 1) / G; ++i) {
+                const int j = gl + G * i;
+                if (j < kMoments / 2) cp_async16(&sums[2 * j], &a.acc[(size_t)c * kMoments + 2 * j]);
+            }
+        cp_async_commit();
+        if constexpr (MODE == MODE_FUSED)
+#pragma unroll
+            for (int i = 0; i < (NOFF + G - 1) / G; ++i)
+                if (gl + G * i < NOFF) dest[gl + G * i] = make_uint2(0u, 0u);
+        // B. the collisions
+        ntc_collisions<Real, NB>(cand, a.seed, gc, s, n, nsel, va + 2, vb, perm, grp, gl, cm, ncoll, flags);
         if (has_r && gl == 0) a.crmax[c] = cm;
+        __syncwarp();
         // C. moment sums of the collided particles; the cell is written back in place in
         // stable order (the collide, and cells the step's LB2DSMC regenerates), or moved on.
         // Every lane sums its particles gl, gl + G, gl + 2 G, ... in this order, whether in
@@ -611,42 +613,74 @@ __device__ __forceinline__ void collide_warp(const DsmcArgs<Real>& a, uint32_t p
         Real mo[kMoments];
 #pragma unroll
         for (int q = 0; q < kMoments; ++q) mo[q] = (Real)0;
-        const bool back = has_r && !moving;
-        const uint32_t nback = back ? n : 0u;
-        for (uint32_t k = gl; k < nback; k += G) {
-            const Real ux = vx[k], uy = vy[k], uz = vz[k];
-            rec_put(a.drec, base + k, qx[k], qy[k], Z3 ? qz[k] : (Real)0, ux, uy, uz, 0u);
+        const uint32_t nback = has_r && !moving ? n : 0u;
+        const uint32_t backmax = MODE == MODE_FUSED ? __reduce_max_sync(kFull, nback) : nmax;
+#pragma unroll 1
+        for (uint32_t k0 = 0; k0 < backmax; k0 += G) {
+            const uint32_t k = k0 + (uint32_t)gl;
+            if (k >= nback) continue;
+            const uint32_t p = perm[k];
+            Real px, py, ux, uy;
+            get4(va + 4 * p, px, py, ux, uy);
+            const Real uz = vb[NB * p];
+            rec_put(a.drec, base + k, px, py, Z3 ? vb[NB * p + NB - 1] : (Real)0, ux, uy, uz, 0u);
             if (do_sample) add_moments(mo, ux, uy, uz);
         }
+        // the move of step s + 1 in place in the pool: every particle takes its place among those
+        // of its cell bound for the same neighbour from a shared count
+        const uint32_t nm = moving && act ? n : 0u;
+        constexpr int NO = (NOFF + G - 1) / G;
+        uint32_t to[NO], at[NO], many[NO];
         if constexpr (MODE == MODE_FUSED) {
-            // the move of step s + 1, straight from the pool: particle k of cell c, one per
-            // lane at a time, into the bins of half p with its order key
             const MoveCtx<Real> m = move_ctx(a);
             const Origin org = origin_of(m, gc);
             const Half<Real> dst = half_s(a);
-            const uint32_t nm = moving && act ? n : 0u;
-            const uint32_t nmax = __reduce_max_sync(kFull, nm);
+#pragma unroll 1
             for (uint32_t k0 = 0; k0 < nmax; k0 += G) {
-                const uint32_t k1 = k0 + (uint32_t)gl;
-                const bool act1 = k1 < nm;
-                Real p1[6] = {0, 0, 0, 0, 0, 0};
-                if (act1) {
-                    p1[0] = qx[k1]; p1[1] = qy[k1]; if constexpr (Z3) p1[2] = qz[k1];
-                    p1[3] = vx[k1]; p1[4] = vy[k1]; p1[5] = vz[k1];
-                    if (do_sample) add_moments(mo, p1[3], p1[4], p1[5]);
-                }
-                uint32_t key1 = 0, ok1 = 0;
-                int dir1 = -1;
-                if (act1)  // (multi-step calls run on whole channels: no particle leaves)
-                    key1 = move_particle<Real, Z3, false>(m, org, k1, s + 1u, p1[0], p1[1], p1[2], p1[3], p1[4],
-                                                          p1[5], hits, caps, dir1, ok1);
-                const uint32_t arr1 = bin_arrival1(dst.count, key1, act1, lane);
-                if (act1) {
-                    if (arr1 < bin)
-                        put_particle<Real, Z3>(dst, (int64_t)key1 * bin + arr1, ok1, p1[0], p1[1], p1[2],
-                                               p1[3], p1[4], p1[5]);
+                const uint32_t k = k0 + (uint32_t)gl;
+                if (k >= nm) continue;
+                const uint32_t p = perm[k];
+                Real px, py, pz = 0, ux, uy, uz = vb[NB * p];
+                get4(va + 4 * p, px, py, ux, uy);
+                if constexpr (Z3) pz = vb[NB * p + NB - 1];
+                if (do_sample) add_moments(mo, ux, uy, uz);
+                int ix, iy, iz;
+                fly<Real, Z3>(m, org, k, s + 1u, px, py, pz, ux, uy, uz, hits, caps, ix, iy, iz);
+                const uint32_t o = neighbour_offset<Real, Z3>(m, org, ix, iy, iz);
+                if (o != kFarOffset) {
+                    key[p] = (o << 16) | atomicAdd(&dest[o].x, 1u);
+                    put4(va + 4 * p, px, py, ux, uy);
+                    vb[NB * p] = uz;
+                    if constexpr (Z3) vb[NB * p + NB - 1] = pz;
+                } else {  // farther than a neighbour: put away at once
+                    key[p] = 0xFFFFFFFFu;
+                    const uint32_t cell = (uint32_t)((iz * a.ncy + iy) * a.ncx + ix);
+                    const uint32_t arr = atomicAdd(&dst.count[cell], 1u);
+                    if (arr < bin)
+                        put_particle<Real, Z3>(dst, (int64_t)cell * bin + arr, order_key(m, org, k, o), px, py, pz,
+                                               ux, uy, uz);
                     else
                         lost += 1;
+                }
+            }
+            __syncwarp();
+            // one reservation of slots per neighbour, all of a cell's in flight together
+#pragma unroll
+            for (int i = 0; i < NO; ++i) {
+                const int o = gl + G * i;
+                many[i] = o < NOFF && moving && act ? dest[o].x : 0u;
+                to[i] = at[i] = 0u;
+                if (many[i] > 0u) {
+                    int x = org.x + o % 3 - 1, y = org.y + (o / 3) % 3 - 1, z = 0;
+                    if (y < 0) y += m.ncy;
+                    if (y >= m.ncy) y -= m.ncy;
+                    if constexpr (Z3) {
+                        z = org.z + o / 9 - 1;
+                        if (z < 0) z += m.ncz;
+                        if (z >= m.ncz) z -= m.ncz;
+                    }
+                    to[i] = (uint32_t)((z * m.ncy + y) * m.ncx + x);
+                    at[i] = atomicAdd(&dst.count[to[i]], many[i]);
                 }
             }
             // the arrivals of half p^1 are consumed: their count starts the next step's
@@ -678,7 +712,32 @@ __device__ __forceinline__ void collide_warp(const DsmcArgs<Real>& a, uint32_t p
 #pragma unroll
                 for (int q = 0; q < 3; ++q) {
                     const int mq = 3 * gl + q;
-                    if (mq < kMoments) a.acc[(size_t)c * kMoments + mq] = sums[mq] + widen(t[q]);
+                    if (mq < kMoments) a.acc[(size_t)c * kMoments + mq] = sums[mq] + (double)t[q];
+                }
+            }
+        }
+        if constexpr (MODE == MODE_FUSED) {
+            const Half<Real> dst = half_s(a);
+#pragma unroll
+            for (int i = 0; i < NO; ++i)
+                if (gl + G * i < NOFF)
+                    dest[gl + G * i] = make_uint2(to[i] * bin + at[i], at[i] < bin ? bin - at[i] : 0u);
+            __syncwarp();
+#pragma unroll 1
+            for (uint32_t k0 = 0; k0 < nmax; k0 += G) {
+                const uint32_t k = k0 + (uint32_t)gl;
+                if (k >= nm) continue;
+                const uint32_t p = perm[k], w = key[p];
+                if (w != 0xFFFFFFFFu) {
+                    const uint32_t o = w >> 16, r = w & 0xFFFFu;
+                    const uint2 d = dest[o];
+                    Real px, py, ux, uy;
+                    get4(va + 4 * p, px, py, ux, uy);
+                    if (r < d.y)
+                        put_particle<Real, Z3>(dst, (int64_t)(d.x + r), o * bin + k, px, py,
+                                               Z3 ? vb[NB * p + NB - 1] : (Real)0, ux, uy, vb[NB * p]);
+                    else
+                        lost += 1;
                 }
             }
         }
@@ -914,7 +973,7 @@ cudaError_t collide_impl_w(Ctx& c, int p) {
     c.cur_p = save;
     constexpr int NC = W * kWarpCells;
     const uint32_t pool = collide_pool(c);
-    const uint32_t warp_smem = collide_warp_smem<Real, Z3>(pool, (uint32_t)c.d.bin);
+    const uint32_t warp_smem = warp_mem<Real, Z3>(pool, (uint32_t)c.d.bin).total;
     const size_t smem = (size_t)W * warp_smem;
     // (dynamic and static shared memory together may exceed the default 48 KB)
     cudaError_t e = cudaFuncSetAttribute(k_collide<Real, false, Z3, MODE, W>,
@@ -1055,14 +1114,14 @@ bool fused_fills_gpu_w(const Ctx& c) {
     int per_sm;
     if (c.p.real_bytes == 4)
         per_sm = z3 ? collide_per_sm(k_collide<float, false, true, MODE_FUSED, W>, W * 32,
-                                     (size_t)W * collide_warp_smem<float, true>(pool, bin))
+                                     (size_t)W * warp_mem<float, true>(pool, bin).total)
                     : collide_per_sm(k_collide<float, false, false, MODE_FUSED, W>, W * 32,
-                                     (size_t)W * collide_warp_smem<float, false>(pool, bin));
+                                     (size_t)W * warp_mem<float, false>(pool, bin).total);
     else
         per_sm = z3 ? collide_per_sm(k_collide<double, false, true, MODE_FUSED, W>, W * 32,
-                                     (size_t)W * collide_warp_smem<double, true>(pool, bin))
+                                     (size_t)W * warp_mem<double, true>(pool, bin).total)
                     : collide_per_sm(k_collide<double, false, false, MODE_FUSED, W>, W * 32,
-                                     (size_t)W * collide_warp_smem<double, false>(pool, bin));
+                                     (size_t)W * warp_mem<double, false>(pool, bin).total);
     if (per_sm < 1) return true;
     const int64_t blocks = (c.d.ncells + NC - 1) / NC;
     return blocks >= (int64_t)per_sm * c.num_sms;
@@ -1103,7 +1162,7 @@ cudaError_t batch_collide_impl(BatchDev& b, int cur_p) {
     L.tab = (const DsmcArgs<Real>*)b.dsmc[cur_p];
     L.nrep = b.nrep;
     cudaError_t e;
-    const uint32_t warp_smem = collide_warp_smem<Real, false>(b.pool, b.maxbin);
+    const uint32_t warp_smem = warp_mem<Real, false>(b.pool, b.maxbin).total;
     const size_t smem = (size_t)(b.collide_block / 32) * warp_smem;
     if (b.collide_block == 128) {  // blocks of 16 cells
         L.pre = b.pre_blocks4;
