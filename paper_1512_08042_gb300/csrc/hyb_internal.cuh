@@ -143,9 +143,9 @@ struct LbmArgs {
 };
 
 // One step of the adjoint of the LBM with per-node parameters: lam_next = dL/df_{t+1} in,
-// lam = dL/df_t out, the parameter gradients accumulated; wall = 2 ny adjoint wall
-// densities (left rows, then right rows) followed by a 32-bit block ticket, all zero on entry
-// and left zero.
+// lam = dL/df_t out, the parameter gradients accumulated. A row of nx nodes is cut into nseg
+// segments of `width` (at most 32) nodes, a warp each. early: the populations at t were complete
+// before the previous kernel of the stream began its work.
 template <typename Real>
 struct LbmAdjArgs {
     const Real* f;         // populations at t
@@ -155,8 +155,8 @@ struct LbmAdjArgs {
     const Real* tau_node;
     Real* grad_g;
     Real* grad_tau;
-    Real* wall;  // 2 nrows wall sums (left, right; row z ny + y) and a ticket
     int32_t nx, ny, nz;
+    int32_t nseg, width, early;
     int64_t nnodes;
 };
 
@@ -266,6 +266,13 @@ __device__ __forceinline__ int replica_of(const int64_t* pre, int nrep, int64_t 
 __device__ __forceinline__ void pdl_begin() {
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+
+// For kernels whose next one may read, before its own wait, what was complete before this kernel
+// began its work: the next kernel is scheduled only once this one's wait is over.
+__device__ __forceinline__ void pdl_after_wait() {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
 
 // Asynchronous 16-byte copies from global to shared memory (cp.async, sm_80 and later),
@@ -515,7 +522,7 @@ cudaError_t launch_lbm_halo(Ctx& c, int side, void* buf, int unpack);
 cudaError_t launch_lbm_step_nodes(Ctx& c, const void* f_src, void* f_dst, const void* g, const void* tau);
 cudaError_t launch_lbm_adjoint_step(Ctx& c, const void* f, const void* lam_next, void* lam,
                                     const void* g, const void* tau, void* grad_g, void* grad_tau,
-                                    void* wall);
+                                    bool early);
 cudaError_t launch_interface_loss(Ctx& c, const void* f, const int32_t* nodes, int32_t n,
                                   const void* targets, double* loss, void* lam);
 cudaError_t launch_map_d2l(Ctx& c, const int32_t* nodes, int32_t n);

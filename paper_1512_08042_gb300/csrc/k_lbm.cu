@@ -317,6 +317,7 @@ __global__ void __launch_bounds__(128) k_lbm(Launch<LbmArgs<Real>> L) {
 // One thread per node, with per-node force increment and relaxation time.
 template <typename Real, class LAT, bool BGK, bool Z3 = false>
 __global__ void __launch_bounds__(128) k_lbm_param(LbmArgs<Real> a) {
+    pdl_after_wait();
     const int64_t u = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (u < a.nnodes) lbm_node<Real, LAT, true, BGK, Z3>(a, u);
 }
@@ -330,8 +331,8 @@ __global__ void __launch_bounds__(128) k_lbm_param(LbmArgs<Real> a) {
 // populations -> combined coefficients (A0, A1, A2, B3) -> (rho, u, P, Q3, g, om, of) ->
 // raw moments -> streamed populations. P^T is a permutation: mu_q(x) goes to
 // lam_t[q](x - e_q), except for sources behind a wall, whose mu feeds the wall density of
-// the row (summed in `wall` and spread over the populations leaving through that wall by
-// the last block of k_lbm_adj).
+// the row (summed by the warp next to the wall and spread over the populations leaving through
+// it).
 
 // Third-order terms of B3[k] (k = xxx xxy xxz xyy xyz xzz yyy yyz yzz zzz):
 //   B3[k] = rho M_k(u) + om (Q3_k - rho (M_k + L_k(u)) - kap_k a1y) + of rho g f_k(u),
@@ -376,24 +377,51 @@ __device__ __forceinline__ void b3_terms(int k, Real ux, Real uy, Real uz, Real&
     }
 }
 
+// The raw moments of a node's streamed populations at step t (the forward intermediates that
+// the adjoint starts from).
+template <typename Real>
+struct NodeMoments {
+    Real rho, jx, jy, jz, pm[6], q3[10];
+};
 template <typename Real, class LAT, bool Z3>
-__device__ __forceinline__ void lbm_adjoint_node(const LbmAdjArgs<Real>& a, const int64_t node) {
+__device__ __forceinline__ void adjoint_moments(const LbmAdjArgs<Real>& a, int x, int y, int z, NodeMoments<Real>& m) {
+    Real fs[LAT::Q];
+    if constexpr (Z3)
+        pull_node<Real, LAT, true>(a.f, x, y, a.nx, a.ny, a.nnodes, fs, z, a.nz);
+    else
+        pull_node<Real, LAT>(a.f, x, y, a.nx, a.ny, a.nnodes, fs);
+    node_moments<Real, LAT>(fs, m.rho, m.jx, m.jy, m.jz, m.pm, m.q3);
+}
+
+// The parts of a row's wall adjoint: one per population entering through the wall and node it
+// would have come past (the sum of the positive e_x), in ascending (population, x).
+template <class LAT>
+__host__ __device__ constexpr int wall_parts() {
+    int n = 0;
+    for (int q = 0; q < LAT::Q; ++q) n += E<LAT>(q, 0) > 0 ? E<LAT>(q, 0) : 0;
+    return n;
+}
+template <class LAT>
+__host__ __device__ constexpr int wall_part(int q) {  // the first part of population q
+    int n = 0;
+    for (int p = 0; p < q; ++p)
+        if (E<LAT>(p, 0) * E<LAT>(q, 0) > 0) n += E<LAT>(p, 0) > 0 ? E<LAT>(p, 0) : -E<LAT>(p, 0);
+    return n;
+}
+
+// The adjoint of node (x, y, z) from its forward moments; the node's parts of the adjoints of the
+// left and right wall densities of its row go to wl and wr.
+template <typename Real, class LAT, bool Z3>
+__device__ __forceinline__ void lbm_adjoint_node(const LbmAdjArgs<Real>& a, int x, int y, int z,
+                                                 const NodeMoments<Real>& nm, Real* wl, Real* wr) {
     constexpr int Q = LAT::Q;
     constexpr double R = lat_r<LAT>();
     const int nx = a.nx, ny = a.ny;
-    const int x = (int)(node % nx);
-    const int y = Z3 ? (int)((node / nx) % ny) : (int)(node / nx);
-    const int z = Z3 ? (int)(node / ((int64_t)nx * ny)) : 0;
     const int64_t nn = a.nnodes;
-
-    // forward intermediates of the node at t
-    Real fs[Q];
-    if constexpr (Z3)
-        pull_node<Real, LAT, true>(a.f, x, y, nx, ny, nn, fs, z, a.nz);
-    else
-        pull_node<Real, LAT>(a.f, x, y, nx, ny, nn, fs);
-    Real rho, jx, jy, jz, pm[6], q3[10];
-    node_moments<Real, LAT>(fs, rho, jx, jy, jz, pm, q3);
+    const int64_t node = (Z3 ? (int64_t)z * ny + y : (int64_t)y) * nx + x;
+    const Real rho = nm.rho, jx = nm.jx, jy = nm.jy, jz = nm.jz;
+    const Real(&pm)[6] = nm.pm;
+    const Real(&q3)[10] = nm.q3;
     const Real gy = a.g_node[node];
     const Real tau = a.tau_node[node];
     const Real om = (Real)1 - (Real)1 / tau, of = (Real)1 - (Real)0.5 / tau;
@@ -517,7 +545,6 @@ __device__ __forceinline__ void lbm_adjoint_node(const LbmAdjArgs<Real>& a, cons
     a.grad_tau[node] += (omb + (Real)0.5 * ofb) / (tau * tau);
 
     // mu_q = d rho/dfs_q rhob + ... (the moments are sums over q), then P^T
-    constexpr int MV = LAT::MAXV;
     static_for<Q>([&](auto qc) {
         constexpr int q = decltype(qc)::value;
         constexpr int ex = E<LAT>(q, 0), ey = E<LAT>(q, 1), ez = E<LAT>(q, 2);
@@ -543,68 +570,82 @@ __device__ __forceinline__ void lbm_adjoint_node(const LbmAdjArgs<Real>& a, cons
             int64_t srow = wrap_y(y - ey, ny);  // the source row (z - ez) ny + (y - ey)
             if constexpr (Z3) srow += (int64_t)wrap_y(z - ez, a.nz) * ny;
             a.lam[(int64_t)q * nn + srow * nx + sx] = mu;
-        } else if constexpr (ex != 0) {
+        } else if constexpr (ex > 0) {
             // a source behind a wall: fs_q = w_q rho_wall(row (y, z))
-            const int64_t nrows = Z3 ? (int64_t)ny * a.nz : (int64_t)ny;
-            const int64_t row = Z3 ? (int64_t)z * ny + y : (int64_t)y;
-            atomicAdd(&a.wall[(sx < 0 ? 0 : nrows) + row], (Real)W<LAT>(q) * mu);
+            wl[wall_part<LAT>(q) + x] = (Real)W<LAT>(q) * mu;
+        } else if constexpr (ex < 0) {
+            wr[wall_part<LAT>(q) + x - (nx + ex)] = (Real)W<LAT>(q) * mu;
         }
     });
-    (void)MV;
 }
 
-// The populations leaving through a wall on row (y', z') feed the wall density of row
-// (y' + e_y, z' + e_z); their adjoint is that row's wall adjoint times the flux
-// normalisation. Task t < 2 nrows: the left (t < nrows) or right wall of source row
-// z' ny + y' (z' = 0 for the slab). The wall sums are read from L2.
-template <typename Real, class LAT, bool Z3>
-__device__ __forceinline__ void adj_wall_row(const LbmAdjArgs<Real>& a, int64_t t) {
-    const int ny = a.ny, nx = a.nx;
-    const int64_t nrows = Z3 ? (int64_t)ny * a.nz : (int64_t)ny;
-    const bool left = t < nrows;
-    const int64_t r = left ? t : t - nrows;  // the source row
-    const int yr = (int)(r % ny), zr = (int)(r / ny);
+// The wall adjoint from its parts, added one after another (no contraction with their products).
+template <class LAT>
+__device__ __forceinline__ float wall_sum(const float* parts) {
+    float s = 0.f;
+#pragma unroll
+    for (int i = 0; i < wall_parts<LAT>(); ++i) s = __fadd_rn(s, parts[i]);
+    return s;
+}
+template <class LAT>
+__device__ __forceinline__ double wall_sum(const double* parts) {
+    double s = 0.0;
+#pragma unroll
+    for (int i = 0; i < wall_parts<LAT>(); ++i) s = __dadd_rn(s, parts[i]);
+    return s;
+}
+
+// The populations that leave through a wall from row (y - e_y, z - e_z) feed the wall density of
+// row (y, z); their adjoint is that row's wall adjoint wb times the flux normalisation. No node
+// writes them.
+template <typename Real, class LAT, bool Z3, bool LEFT>
+__device__ __forceinline__ void adjoint_wall_row(const LbmAdjArgs<Real>& a, int y, int z, Real wb) {
     constexpr double inv_flux = 1.0 / wall_flux_norm<LAT>();
+    const Real v = (Real)inv_flux * wb;
     static_for<LAT::Q>([&](auto qc) {
         constexpr int q = decltype(qc)::value;
         constexpr int ex = E<LAT>(q, 0), ey = E<LAT>(q, 1), ez = E<LAT>(q, 2);
-        if constexpr (ex != 0) {
-            if ((ex < 0) == left) {
-                int64_t drow = wrap_y(yr + ey, ny);
-                if constexpr (Z3) drow += (int64_t)wrap_y(zr + ez, a.nz) * ny;
-                const Real wb = (Real)inv_flux * __ldcg(&a.wall[(left ? 0 : nrows) + drow]);
-                Real* lq = a.lam + (int64_t)q * a.nnodes + r * nx;
-                if (ex < 0)
-                    for (int i = 0; i < -ex; ++i) lq[i] = wb;
-                else
-                    for (int i = nx - ex; i < nx; ++i) lq[i] = wb;
-            }
+        if constexpr (LEFT ? ex < 0 : ex > 0) {
+            int64_t srow = wrap_y(y - ey, a.ny);
+            if constexpr (Z3) srow += (int64_t)wrap_y(z - ez, a.nz) * a.ny;
+            Real* lq = a.lam + (int64_t)q * a.nnodes + srow * a.nx + (LEFT ? 0 : a.nx - ex);
+#pragma unroll
+            for (int i = 0; i < (LEFT ? -ex : ex); ++i) lq[i] = v;
         }
     });
 }
 
-// One thread per node: the collision adjoint and the transposed pull. The last block to
-// finish (a ticket after the wall sums of every block) spreads the wall adjoints over the
-// populations leaving through the walls, which no node writes, and clears the sums.
+// One thread per node: the collision adjoint and the transposed pull. A row is cut into segments
+// of equal width, at most 32 nodes, a warp each, so that the nodes next to a wall (as many as the
+// largest speed, three at most, and a row has at least six) are in one warp, which adds up the
+// row's wall adjoint and writes the populations it feeds. Bound by latency at 256 x 128 nodes (1.7
+// warps per scheduler). There the last block of a grid-wide ticket, which spread the sums of every
+// row, ran alone for half of the kernel's time: a gradient of 100 steps took 3.58 ms, of which the
+// adjoint 24.7 us a step; without the tail and with the launches overlapped 2.09 ms.
+// With `early` the populations at t are known to be complete when the previous kernel of the
+// stream starts its work, and the forward moments are formed before that kernel has finished: the
+// next kernel may only be scheduled once this one's wait is over (launch_dependents after the
+// wait), so at most the previous kernel is still running then.
 template <typename Real, class LAT, bool Z3 = false>
 __global__ void __launch_bounds__(128) k_lbm_adj(LbmAdjArgs<Real> a) {
-    __shared__ int s_last;
-    const int64_t u = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (u < a.nnodes) lbm_adjoint_node<Real, LAT, Z3>(a, u);
-    __syncthreads();
-    const int64_t nrows = Z3 ? (int64_t)a.ny * a.nz : (int64_t)a.ny;
-    unsigned* ticket = reinterpret_cast<unsigned*>(a.wall + 2 * nrows);
-    if (threadIdx.x == 0) {
-        __threadfence();  // this block's wall sums are visible before its ticket
-        s_last = atomicAdd(ticket, 1u) == gridDim.x - 1u;
-    }
-    __syncthreads();
-    if (!s_last) return;
-    __threadfence();
-    for (int64_t t = threadIdx.x; t < 2 * nrows; t += blockDim.x) adj_wall_row<Real, LAT, Z3>(a, t);
-    __syncthreads();
-    for (int64_t t = threadIdx.x; t < 2 * nrows; t += blockDim.x) a.wall[t] = (Real)0;
-    if (threadIdx.x == 0) *ticket = 0u;
+    const int wid = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5);
+    const int row = wid / a.nseg, seg = wid - row * a.nseg;
+    const unsigned lane = lane_id();
+    const int x0 = seg * a.width, x = x0 + (int)lane;
+    const int y = Z3 ? row % a.ny : row, z = Z3 ? row / a.ny : 0;
+    const bool act = row < a.ny * a.nz && (int)lane < a.width && x < a.nx;
+    NodeMoments<Real> nm;
+    if (a.early && act) adjoint_moments<Real, LAT, Z3>(a, x, y, z, nm);
+    pdl_after_wait();
+    if (row >= a.ny * a.nz) return;  // whole warps
+    if (!a.early && act) adjoint_moments<Real, LAT, Z3>(a, x, y, z, nm);
+    __shared__ Real s_wall[4][2][wall_parts<LAT>()];
+    Real* wl = s_wall[(threadIdx.x >> 5) & 3][0];
+    Real* wr = s_wall[(threadIdx.x >> 5) & 3][1];
+    if (act) lbm_adjoint_node<Real, LAT, Z3>(a, x, y, z, nm, wl, wr);
+    __syncwarp();
+    if (x0 == 0 && lane == 0) adjoint_wall_row<Real, LAT, Z3, true>(a, y, z, wall_sum<LAT>(wl));
+    if (x0 + a.width >= a.nx && lane == 31) adjoint_wall_row<Real, LAT, Z3, false>(a, y, z, wall_sum<LAT>(wr));
 }
 
 // Packed index of the symmetric pair (i, j): xx xy xz yy yz zz.
@@ -743,12 +784,12 @@ LbmArgs<Real> lbm_args(const Ctx& c, int cur_f) {
 template <typename Real, class LAT>
 cudaError_t lbm_impl(Ctx& c) {
     const LbmArgs<Real> a = lbm_args<Real>(c, c.cur_f);
-    const int64_t blocks = (c.d.nnodes + 127) / 128;
+    const unsigned block = 128;
     prof_begin(c, K_LBM);
     Launch<LbmArgs<Real>> L{};
     L.one = a;
     L.total = c.d.nnodes;
-    const dim3 g((unsigned)blocks), b(128);
+    const dim3 g((unsigned)((c.d.nnodes + block - 1) / block)), b(block);
     cudaError_t e;
     if (a.nz > 1)  // 3D: periodic in z
         e = a.tau_node ? (a.bgk ? launch_pdl(k_lbm<Real, LAT, false, true, true, true>, g, b, 0, c.stream, L)
@@ -783,23 +824,17 @@ cudaError_t lbm_nodes_impl(Ctx& c, const void* f_src, void* f_dst, const void* g
     a.dst = (Real*)f_dst;
     a.g_node = (const Real*)g;
     a.tau_node = (const Real*)tau;
-    const int64_t blocks = (c.d.nnodes + 127) / 128;
-    if (a.nz > 1) {
-        if (a.bgk)
-            k_lbm_param<Real, LAT, true, true><<<(unsigned)blocks, 128, 0, c.stream>>>(a);
-        else
-            k_lbm_param<Real, LAT, false, true><<<(unsigned)blocks, 128, 0, c.stream>>>(a);
-    } else if (a.bgk) {
-        k_lbm_param<Real, LAT, true><<<(unsigned)blocks, 128, 0, c.stream>>>(a);
-    } else {
-        k_lbm_param<Real, LAT, false><<<(unsigned)blocks, 128, 0, c.stream>>>(a);
-    }
-    return cudaGetLastError();
+    const dim3 grid((unsigned)((c.d.nnodes + 127) / 128)), b(128);
+    if (a.nz > 1)
+        return a.bgk ? launch_pdl(k_lbm_param<Real, LAT, true, true>, grid, b, 0, c.stream, a)
+                     : launch_pdl(k_lbm_param<Real, LAT, false, true>, grid, b, 0, c.stream, a);
+    return a.bgk ? launch_pdl(k_lbm_param<Real, LAT, true>, grid, b, 0, c.stream, a)
+                 : launch_pdl(k_lbm_param<Real, LAT, false>, grid, b, 0, c.stream, a);
 }
 
 template <typename Real, class LAT>
 cudaError_t lbm_adj_impl(Ctx& c, const void* f, const void* lam_next, void* lam, const void* g,
-                         const void* tau, void* grad_g, void* grad_tau, void* wall) {
+                         const void* tau, void* grad_g, void* grad_tau, bool early) {
     LbmAdjArgs<Real> a;
     a.f = (const Real*)f;
     a.lam_next = (const Real*)lam_next;
@@ -808,17 +843,17 @@ cudaError_t lbm_adj_impl(Ctx& c, const void* f, const void* lam_next, void* lam,
     a.tau_node = (const Real*)tau;
     a.grad_g = (Real*)grad_g;
     a.grad_tau = (Real*)grad_tau;
-    a.wall = (Real*)wall;
     a.nx = (int32_t)c.d.nx;
     a.ny = (int32_t)c.d.ny;
     a.nz = (int32_t)c.d.nz;
     a.nnodes = c.d.nnodes;
-    const int64_t blocks = (c.d.nnodes + 127) / 128;
-    if (a.nz > 1)
-        k_lbm_adj<Real, LAT, true><<<(unsigned)blocks, 128, 0, c.stream>>>(a);
-    else
-        k_lbm_adj<Real, LAT><<<(unsigned)blocks, 128, 0, c.stream>>>(a);
-    return cudaGetLastError();
+    a.nseg = (a.nx + 31) / 32;
+    a.width = (a.nx + a.nseg - 1) / a.nseg;
+    a.early = early ? 1 : 0;
+    const int64_t warps = (int64_t)a.nseg * a.ny * a.nz;
+    const dim3 grid((unsigned)((warps + 3) / 4)), b(128);  // (32 or 64 threads: 8% or 2% slower)
+    return a.nz > 1 ? launch_pdl(k_lbm_adj<Real, LAT, true>, grid, b, 0, c.stream, a)
+                    : launch_pdl(k_lbm_adj<Real, LAT>, grid, b, 0, c.stream, a);
 }
 
 template <typename Real, class LAT>
@@ -960,14 +995,14 @@ cudaError_t launch_lbm_step_nodes(Ctx& c, const void* f_src, void* f_dst, const 
 
 cudaError_t launch_lbm_adjoint_step(Ctx& c, const void* f, const void* lam_next, void* lam,
                                     const void* g, const void* tau, void* grad_g, void* grad_tau,
-                                    void* wall) {
+                                    bool early) {
     if (c.p.lattice == 39)
         return c.p.real_bytes == 4
-                   ? lbm_adj_impl<float, D3Q39>(c, f, lam_next, lam, g, tau, grad_g, grad_tau, wall)
-                   : lbm_adj_impl<double, D3Q39>(c, f, lam_next, lam, g, tau, grad_g, grad_tau, wall);
+                   ? lbm_adj_impl<float, D3Q39>(c, f, lam_next, lam, g, tau, grad_g, grad_tau, early)
+                   : lbm_adj_impl<double, D3Q39>(c, f, lam_next, lam, g, tau, grad_g, grad_tau, early);
     return c.p.real_bytes == 4
-               ? lbm_adj_impl<float, D3Q19>(c, f, lam_next, lam, g, tau, grad_g, grad_tau, wall)
-               : lbm_adj_impl<double, D3Q19>(c, f, lam_next, lam, g, tau, grad_g, grad_tau, wall);
+               ? lbm_adj_impl<float, D3Q19>(c, f, lam_next, lam, g, tau, grad_g, grad_tau, early)
+               : lbm_adj_impl<double, D3Q19>(c, f, lam_next, lam, g, tau, grad_g, grad_tau, early);
 }
 
 cudaError_t launch_interface_loss(Ctx& c, const void* f, const int32_t* nodes, int32_t n,

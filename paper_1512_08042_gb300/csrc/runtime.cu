@@ -608,7 +608,7 @@ hyb_status lbm_adjoint_step(hyb_ctx* h, const void* f, const void* lam_next, voi
         !grad_tau || !wall || h->c.p.lb_collision != 0)
         return HYB_EINVAL;
     return check(h->c, launch_lbm_adjoint_step(h->c, f, lam_next, lam, g_node, tau_node, grad_g,
-                                               grad_tau, wall),
+                                               grad_tau, false),
                  "lbm_adjoint_step launch");
 }
 
@@ -655,8 +655,9 @@ hyb_status lbm_adjoint_segment(hyb_ctx* h, const void* state0, void* states, int
     void* next = lam_a;
     void* cur = lam_b;
     for (int32_t k = n - 1; k >= 0; --k) {
+        // state k was complete before adjoint step k + 1, the previous kernel, began its work
         hyb_status s = check(c, launch_lbm_adjoint_step(c, state(k), next, cur, g_node, tau_node, grad_g,
-                                                        grad_tau, wall),
+                                                        grad_tau, k < n - 1),
                              "lbm_adjoint_segment step");
         if (s != HYB_OK) return s;
         std::swap(next, cur);
