@@ -182,13 +182,19 @@ __device__ __forceinline__ Real wrap_periodic(Real v, Real period) {
 // Kick (v_y += g), then the flight of one step from (px, py, pz) with walls and periodic
 // wrap, of the particle of rank k of the channel's cell o at the start of step s (the key of its
 // wall draws); its new column, channel row and layer.
-template <typename Real, bool Z3>
+// WALLS = false: a particle whose straight flight stays between the walls (flies_straight).
+template <typename Real>
+__device__ __forceinline__ bool flies_straight(const MoveCtx<Real>& m, Real px, Real ux) {
+    const Real xn = px + ux * m.dt;
+    return xn >= (Real)0 && xn <= m.H;
+}
+template <typename Real, bool Z3, bool WALLS = true>
 __device__ __forceinline__ void fly(const MoveCtx<Real>& m, const Origin& o, uint32_t k, uint32_t s, Real& px,
                                     Real& py, Real& pz, Real& ux, Real& uy, Real& uz, uint32_t& hits,
                                     uint32_t& caps, int& ix, int& iy, int& iz) {
     uy = uy + m.g;
     const Real xn = px + ux * m.dt;
-    if (xn >= (Real)0 && xn <= m.H) {
+    if (!WALLS || (xn >= (Real)0 && xn <= m.H)) {
         px = xn;
         py = py + uy * m.dt;
         if constexpr (Z3) pz = pz + uz * m.dt;
@@ -211,13 +217,13 @@ __device__ __forceinline__ void fly(const MoveCtx<Real>& m, const Origin& o, uin
 // with dir = -1; for a particle that leaves a streamwise slab, the channel's cell
 // (iz ncy + iy) ncx + ix and dir = 0 (towards lower rows) or 1 (higher rows, across the periodic
 // end included). `key` is its order key in the new cell.
-template <typename Real, bool Z3>
+template <typename Real, bool Z3, bool WALLS = true>
 __device__ __forceinline__ uint32_t move_particle(const MoveCtx<Real>& m, const Origin& o, uint32_t k,
                                                   uint32_t s, Real& px, Real& py, Real& pz, Real& ux,
                                                   Real& uy, Real& uz, uint32_t& hits, uint32_t& caps,
                                                   int& dir, uint32_t& key) {
     int ix, iy, iz;
-    fly<Real, Z3>(m, o, k, s, px, py, pz, ux, uy, uz, hits, caps, ix, iy, iz);
+    fly<Real, Z3, WALLS>(m, o, k, s, px, py, pz, ux, uy, uz, hits, caps, ix, iy, iz);
     key = order_key(m, o, k, neighbour_offset<Real, Z3>(m, o, ix, iy, iz));
     const int iyl = iy - m.y0;
     if (iyl >= 0 && iyl < m.nly) {
