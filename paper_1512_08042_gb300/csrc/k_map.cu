@@ -1,7 +1,7 @@
 // The two kinetic mappings of Sec. 2. The Grad/Hermite coefficients are formed in FP64;
 // populations and particle state are Real (float or double).
 //
-// k_d2l (DSMC2LB, Sec. 2.1): one warp per coupling node. The cumulative sums of the
+// k_d2l (DSMC2LB, Sec. 2.1): one warp per one or two coupling nodes. The cumulative sums of the
 // node's DSMC cell give rho = <N>/ppc, the per-particle raw moments <v>, <vv>, <vvv> (one
 // FP64 reciprocal of the count) and the raw Hermite coefficients a0 = rho, a1 = rho <v>,
 // a2 = rho(<vv> - I), a3 = rho(<vvv> - sym(<v> I)), all in FP64 (the stress and heat-flux
@@ -12,8 +12,7 @@
 // LB2DSMC (Sec. 2.2, Table 1), k_l2d: one block per coupling cell. Warp 0 forms, in FP64, the
 // mean populations of the cell's lb_ratio^2 nodes, rho and u, the comoving coefficients
 // a2 = sum f c c / rho - I and a3 = sum f c c c / rho (c = xi - u), M, C = 1 + 30 M (Eq. C)
-// and the particle count floor(rho ppc + U); the other warps wait (trials drawn meanwhile
-// took issue slots from warp 0 and lengthened the path). The cell's trial stream is then
+// and the particle count floor(rho ppc + U). The cell's trial stream is then
 // evaluated 256 trials at a time in the state precision, with the coefficients rounded to
 // it: Box-Muller xi from the unit Maxwellian, accepted when C R <= G(xi),
 // G = 1 + a2:H2/2 + a3:H3/6 (Eq. distr_outeq); the k-th accepted trial becomes the k-th
@@ -74,106 +73,138 @@ __device__ __forceinline__ const LatXi<LAT, Real>& lat_xi() {
     }
 }
 
-// DSMC2LB: one warp per coupling node. Lanes 0-19 read the cell's 20 sums and scale them
-// by one FP64 reciprocal of the particle count; the coefficients (one per lane, state
-// precision) are broadcast and each lane evaluates one or two populations.
+// The axes of raw moment k: of the second moments k = 4 to 9 (xx xy xz yy yz zz) in i and j (third
+// axis 0), of the third moments k = 10 to 19 (xxx xxy xxz xyy xyz xzz yyy yyz yzz zzz) in i, j and
+// l; zeros for other k. Two bits per axis, in constants.
+__device__ __forceinline__ void packed_indices(int k, int& i, int& j, int& l) {
+    // six bits per entry, entry e at bits 6 e: i + 4 j + 16 l
+    constexpr unsigned long long second = 0ull | 4ull << 6 | 8ull << 12 | 5ull << 18 | 9ull << 24 | 10ull << 30;
+    constexpr unsigned long long third = 0ull | 16ull << 6 | 32ull << 12 | 20ull << 18 | 36ull << 24 |
+                                         40ull << 30 | 21ull << 36 | 37ull << 42 | 41ull << 48 | 42ull << 54;
+    unsigned code = 0u;
+    if (k >= 4 && k < 10) code = (unsigned)(second >> (6 * (k - 4))) & 63u;
+    if (k >= 10 && k < 20) code = (unsigned)(third >> (6 * (k - 10))) & 63u;
+    i = (int)(code & 3u);
+    j = (int)((code >> 2) & 3u);
+    l = (int)(code >> 4);
+}
+
+// DSMC2LB by one warp for `per` consecutive list entries. Lanes 0-19 read the cell's 20 sums and
+// scale them by one FP64 reciprocal of the particle count; the coefficients (one per lane, state
+// precision) are broadcast and each lane evaluates one or two populations. Nodes of one cell
+// have the same populations, so entries that follow one another in a cell (two nodes per cell and
+// axis) share the solve, which FP64 bounds (19 cycles per warp instruction and SM): the two
+// divisions run in two lanes of one sequence, and the factors 3 of the diagonal terms in one
+// multiplication.
 template <typename Real, class LAT>
-__device__ __forceinline__ void d2l_entries(const MapArgs<Real>& a, int first, int stride) {
+__device__ __forceinline__ void d2l_entries(const MapArgs<Real>& a, int first, int stride, int per) {
     const LatXi<LAT, Real>& lt = lat_xi<LAT, Real>();
     const Real* sx = lt.x;
     const Real* sw = lt.w;
     const unsigned lane = lane_id();
     const uint32_t S = a.ctrl[CTRL_NSAMPLES];
-    for (int t = first; t < a.n; t += stride) {
-        const int32_t node = a.list[t];
-        if (node < 0 || (int64_t)node >= a.nnodes) {
-            if (lane == 0) atomicOr(&a.ctrl[CTRL_STATUS], HYB_ST_BAD_INPUT);
-            continue;
-        }
-        // node (z ny + y) nx + x lies in cell (iz ncy + iy) ncx + ix (z = 0 in 2D); a slab's
-        // ghost rows (the yh rows below and above its own) belong to no cell of the context
-        const int x = node % a.nx, y = (node / a.nx) % a.ny - a.yh, z = node / (a.nx * a.ny);
-        if (y < 0 || y >= a.ncy * a.lb_ratio) {
-            if (lane == 0) atomicOr(&a.ctrl[CTRL_STATUS], HYB_ST_BAD_INPUT);
-            continue;
-        }
-        const int64_t cell =
-            ((int64_t)(z / a.lb_ratio) * a.ncy + y / a.lb_ratio) * a.ncx + (x / a.lb_ratio);
-        const double* m = a.acc + cell * kMoments;
-        const double mk = lane < (unsigned)kMoments ? m[lane] : 0.0;
-        const double NS = __shfl_sync(kFull, mk, 0);
-        if (S == 0 || !(NS > 0.0)) {
-            if (lane == 0) atomicOr(&a.ctrl[CTRL_STATUS], HYB_ST_BAD_INPUT);
-            continue;
-        }
-        // per-particle moments, lane k: <v> (1-3), <vv> (4-9), <vvv> (10-19), and the raw
-        // Hermite coefficients, in FP64; the reciprocal of the count is formed by one lane
-        double inv = 0.0;
-        if (lane == 0) inv = 1.0 / NS;
-        inv = __shfl_sync(kFull, inv, 0);
-        const double mr = mk * inv;
-        const double rho = NS / ((double)S * (double)a.ppc);
-        const double m1x = __shfl_sync(kFull, mr, 1);
-        const double m1y = __shfl_sync(kFull, mr, 2);
-        const double m1z = __shfl_sync(kFull, mr, 3);
-        double sub = 0.0;
-        switch (lane) {
-            case 4: case 7: case 9: sub = 1.0; break;       // xx yy zz
-            case 10: sub = 3.0 * m1x; break;                // xxx
-            case 11: sub = m1y; break;                      // xxy
-            case 12: sub = m1z; break;                      // xxz
-            case 13: sub = m1x; break;                      // xyy
-            case 15: sub = m1x; break;                      // xzz
-            case 16: sub = 3.0 * m1y; break;                // yyy
-            case 17: sub = m1z; break;                      // yyz
-            case 18: sub = m1y; break;                      // yzz
-            case 19: sub = 3.0 * m1z; break;                // zzz
-            default: break;
-        }
-        double coef = lane == 0 ? rho : rho * (mr - sub);
-        if (a.eq_mode && lane >= 4u && lane < (unsigned)kMoments) {
-            // the local equilibrium of rho and u (Sec. 4, Eq. feq_dsmc): a2 = rho u u,
-            // a3 = rho u u u
-            constexpr int I[16][3] = {{0, 0, -1}, {0, 1, -1}, {0, 2, -1}, {1, 1, -1}, {1, 2, -1},
-                                      {2, 2, -1}, {0, 0, 0}, {0, 0, 1}, {0, 0, 2}, {0, 1, 1},
-                                      {0, 1, 2}, {0, 2, 2}, {1, 1, 1}, {1, 1, 2}, {1, 2, 2},
-                                      {2, 2, 2}};
-            const double uu[3] = {m1x, m1y, m1z};
-            const int* ix = I[lane - 4u];
-            coef = rho * uu[ix[0]] * uu[ix[1]];
-            if (ix[2] >= 0) coef = coef * uu[ix[2]];
-        }
-        const Real coef_r = (Real)coef;
-        Real cf[kMoments];
+    constexpr int NH = (LAT::Q + 31) / 32;
+    for (int t0 = first * per; t0 < a.n; t0 += stride * per) {
+        int64_t have = -1;  // the cell whose populations f holds
+        bool usable = false;
+        Real f[NH];
+        for (int t = t0; t < t0 + per && t < a.n; ++t) {
+            const int32_t node = a.list[t];
+            if (node < 0 || (int64_t)node >= a.nnodes) {
+                if (lane == 0) atomicOr(&a.ctrl[CTRL_STATUS], HYB_ST_BAD_INPUT);
+                continue;
+            }
+            // node (z ny + y) nx + x lies in cell (iz ncy + iy) ncx + ix (z = 0 in 2D); a slab's
+            // ghost rows (the yh rows below and above its own) belong to no cell of the context
+            const int x = node % a.nx, y = (node / a.nx) % a.ny - a.yh, z = node / (a.nx * a.ny);
+            if (y < 0 || y >= a.ncy * a.lb_ratio) {
+                if (lane == 0) atomicOr(&a.ctrl[CTRL_STATUS], HYB_ST_BAD_INPUT);
+                continue;
+            }
+            const int64_t cell =
+                ((int64_t)(z / a.lb_ratio) * a.ncy + y / a.lb_ratio) * a.ncx + (x / a.lb_ratio);
+            if (cell != have) {
+                have = cell;
+                const double* m = a.acc + cell * kMoments;
+                const double mk = lane < (unsigned)kMoments ? m[lane] : 0.0;
+                const double NS = __shfl_sync(kFull, mk, 0);
+                usable = S != 0 && NS > 0.0;
+                if (usable) {
+                    // per-particle moments, lane k: <v> (1-3), <vv> (4-9), <vvv> (10-19), and the
+                    // raw Hermite coefficients, in FP64; lane 0 forms the reciprocal of the count and
+                    // lane 1 the density
+                    double qd = 0.0;
+                    if (lane < 2u) {
+                        const double SP = (double)((unsigned long long)S * (unsigned)a.ppc);
+                        qd = (lane == 0 ? 1.0 : NS) / (lane == 0 ? NS : SP);
+                    }
+                    const double inv = __shfl_sync(kFull, qd, 0), rho = __shfl_sync(kFull, qd, 1);
+                    const double mr = mk * inv;
+                    const double m1x = __shfl_sync(kFull, mr, 1);
+                    const double m1y = __shfl_sync(kFull, mr, 2);
+                    const double m1z = __shfl_sync(kFull, mr, 3);
+                    // what the coefficient subtracts: xx yy zz 1; xxx 3x, xxy y, xxz z, xyy x, xzz x,
+                    // yyy 3y, yyz z, yzz y, zzz 3z
+                    double sub = 0.0;
+                    if (lane == 4u || lane == 7u || lane == 9u) sub = 1.0;
+                    if (lane == 10u || lane == 13u || lane == 15u) sub = m1x;
+                    if (lane == 11u || lane == 16u || lane == 18u) sub = m1y;
+                    if (lane == 12u || lane == 17u || lane == 19u) sub = m1z;
+                    sub = sub * (lane == 10u || lane == 16u || lane == 19u ? 3.0 : 1.0);
+                    double coef = lane == 0 ? rho : rho * (mr - sub);
+                    if (a.eq_mode && lane >= 4u && lane < (unsigned)kMoments) {
+                        // the local equilibrium of rho and u (Sec. 4, Eq. feq_dsmc): a2 = rho u u,
+                        // a3 = rho u u u
+                        int i, j, l;
+                        packed_indices((int)lane, i, j, l);
+                        auto uu = [&](int e) { return e == 0 ? m1x : (e == 1 ? m1y : m1z); };
+                        coef = rho * uu(i) * uu(j);
+                        if (lane >= 10u) coef = coef * uu(l);
+                    }
+                    const Real coef_r = (Real)coef;
+                    Real cf[kMoments];
 #pragma unroll
-        for (int k = 0; k < kMoments; ++k) cf[k] = __shfl_sync(kFull, coef_r, k);
-        const Real* a2 = cf + 4;
-        const Real* a3 = cf + 10;
-        const Real tx = a3[0] + a3[3] + a3[5], ty = a3[1] + a3[6] + a3[8], tz = a3[2] + a3[7] + a3[9];
-        const Real tr2 = a2[0] + a2[3] + a2[5];
+                    for (int k = 0; k < kMoments; ++k) cf[k] = __shfl_sync(kFull, coef_r, k);
+                    const Real* a2 = cf + 4;
+                    const Real* a3 = cf + 10;
+                    const Real tx = a3[0] + a3[3] + a3[5], ty = a3[1] + a3[6] + a3[8], tz = a3[2] + a3[7] + a3[9];
+                    const Real tr2 = a2[0] + a2[3] + a2[5];
 #pragma unroll
-        for (int h = 0; h < (LAT::Q + 31) / 32; ++h) {
-            const int q = (int)lane + 32 * h;
-            if (q < LAT::Q) {
-                const Real X = sx[3 * q], Y = sx[3 * q + 1], Z = sx[3 * q + 2];
-                const Real h2 = a2[0] * X * X + a2[3] * Y * Y + a2[5] * Z * Z - tr2 +
-                                (Real)2 * (a2[1] * X * Y + a2[2] * X * Z + a2[4] * Y * Z);
-                Real sum = cf[0] + cf[1] * X + cf[2] * Y + cf[3] * Z + (Real)0.5 * h2;
-                if (LAT::ORDER >= 3) {
-                    const Real cubic = a3[0] * X * X * X + (Real)3 * a3[1] * X * X * Y +
-                                       (Real)3 * a3[2] * X * X * Z + (Real)3 * a3[3] * X * Y * Y +
-                                       (Real)6 * a3[4] * X * Y * Z + (Real)3 * a3[5] * X * Z * Z +
-                                       a3[6] * Y * Y * Y + (Real)3 * a3[7] * Y * Y * Z +
-                                       (Real)3 * a3[8] * Y * Z * Z + a3[9] * Z * Z * Z;
-                    sum += (cubic - (Real)3 * (tx * X + ty * Y + tz * Z)) * (Real)(1.0 / 6.0);
+                    for (int h = 0; h < NH; ++h) {
+                        const int q = (int)lane + 32 * h;
+                        if (q < LAT::Q) {
+                            const Real X = sx[3 * q], Y = sx[3 * q + 1], Z = sx[3 * q + 2];
+                            const Real h2 = a2[0] * X * X + a2[3] * Y * Y + a2[5] * Z * Z - tr2 +
+                                            (Real)2 * (a2[1] * X * Y + a2[2] * X * Z + a2[4] * Y * Z);
+                            Real sum = cf[0] + cf[1] * X + cf[2] * Y + cf[3] * Z + (Real)0.5 * h2;
+                            if (LAT::ORDER >= 3) {
+                                const Real cubic = a3[0] * X * X * X + (Real)3 * a3[1] * X * X * Y +
+                                                   (Real)3 * a3[2] * X * X * Z + (Real)3 * a3[3] * X * Y * Y +
+                                                   (Real)6 * a3[4] * X * Y * Z + (Real)3 * a3[5] * X * Z * Z +
+                                                   a3[6] * Y * Y * Y + (Real)3 * a3[7] * Y * Y * Z +
+                                                   (Real)3 * a3[8] * Y * Z * Z + a3[9] * Z * Z * Z;
+                                sum += (cubic - (Real)3 * (tx * X + ty * Y + tz * Z)) * (Real)(1.0 / 6.0);
+                            }
+                            f[h] = sw[q] * sum;
+                        }
+                    }
                 }
-                a.f[(int64_t)q * a.nnodes + node] = sw[q] * sum;
+            }
+            if (!usable) {
+                if (lane == 0) atomicOr(&a.ctrl[CTRL_STATUS], HYB_ST_BAD_INPUT);
+                continue;
+            }
+#pragma unroll
+            for (int h = 0; h < NH; ++h) {
+                const int q = (int)lane + 32 * h;
+                if (q < LAT::Q) a.f[(int64_t)q * a.nnodes + node] = f[h];
             }
         }
     }
 }
 
-// DSMC2LB: one warp per listed node (the listed nodes of all replicas in the batch form).
+// DSMC2LB: one warp per lb_ratio listed nodes, or per listed node of all replicas in the batch
+// form.
 template <typename Real, class LAT, bool BATCH>
 __global__ void __launch_bounds__(256) k_d2l(Launch<MapArgs<Real>> L) {
     pdl_begin();
@@ -182,9 +213,9 @@ __global__ void __launch_bounds__(256) k_d2l(Launch<MapArgs<Real>> L) {
         if (gw >= L.total) return;
         const int r = replica_of(L.pre, L.nrep, gw);
         const MapArgs<Real>& a = L.tab[r];
-        d2l_entries<Real, LAT>(a, (int)(gw - L.pre[r]), a.n);
+        d2l_entries<Real, LAT>(a, (int)(gw - L.pre[r]), a.n, 1);
     } else {
-        d2l_entries<Real, LAT>(L.one, (int)gw, (int)(((int64_t)gridDim.x * blockDim.x) >> 5));
+        d2l_entries<Real, LAT>(L.one, (int)gw, (int)(((int64_t)gridDim.x * blockDim.x) >> 5), L.one.lb_ratio);
     }
 }
 
@@ -376,19 +407,10 @@ __device__ __forceinline__ const LatBasis<LAT>& lat_basis() {
         return g_basis19;
 }
 
-// Index pairs and triples of the packed second and third moments.
-__device__ __forceinline__ void packed_pair(int k, int& i, int& j) {
-    constexpr int P[6][2] = {{0, 0}, {0, 1}, {0, 2}, {1, 1}, {1, 2}, {2, 2}};
-    i = P[k][0];
-    j = P[k][1];
-}
+// Position of the pair (i, j) among the packed second moments xx xy xz yy yz zz.
 __device__ __forceinline__ int packed_pair_index(int i, int j) {
-    if (i > j) {
-        const int t = i;
-        i = j;
-        j = t;
-    }
-    return i == 0 ? j : (i == 1 ? 2 + j : 5);
+    const int lo = min(i, j), hi = max(i, j);
+    return lo == 0 ? hi : (lo == 1 ? 2 + hi : 5);
 }
 
 // Table 1 step 1 for the cell `cell`, in FP64 (the Grad-coefficient solve), by the whole
@@ -398,17 +420,24 @@ __device__ __forceinline__ int packed_pair_index(int i, int j) {
 //      nodes summed in FP64;
 //   2. warp w, lane k < 20: the partial raw moment sum_q f_q B_k(xi_q) over the populations
 //      q in [w QW, (w + 1) QW) (fused multiply-adds, q ascending);
-//   3. warp 0, lane k: R_k, the sum of the warps' partials (w ascending), then one comoving
+//   3. warp 0, lane k: R_k, the sum of the warps' partials, then one comoving
 //      coefficient from the raw moments:
 //        u_i = R_i / rho,
 //        a2_ij = R_ij / rho - u_i u_j - d_ij                                 (= sum f c c / rho - d),
 //        a3_ijk = (R_ijk - u_i R_jk - u_j R_ik - u_k R_ij) / rho + 2 u_i u_j u_k (= sum f c c c / rho),
 //      c = xi - u, exact identities of the centred sums.
-// Every thread of the block calls it. Returns, in the lanes of warp 0, the packed FP64 value
-// (lane k < 20 holds value k: a2[6], a3[10], u[3], C = 1 + 30 M) and rho.
-template <typename Real, class LAT, bool Z3>
-__device__ __forceinline__ void grad_coefficients(const MapArgs<Real>& a, int cell, double& mine,
-                                                  double& rho_out) {
+// Every thread of the block calls it. `basis` is the Hermite basis in shared memory. draw_first is
+// called between the loads of the populations and their first use. Returns, in the lanes of
+// warp 0, the packed FP64 value (lane k < 20 holds value k: a2[6], a3[10], u[3], C = 1 + 30 M), and
+// rho and the new particle count floor(rho ppc + ur). Bound by latency: the FP64 chain of warp 0 (66
+// cycles an operation) and the loads before it, so the first trials' draws come between the loads
+// and their use, the basis waits in shared memory, and no table indexed by the lane sits in
+// local memory (with DSMC2LB's shared solves: 20 hybrid steps of 819k particles 1.34 -> 1.25 ms,
+// of 6.55M in 3D with 2048 coupling cells 9.01 -> 8.43 ms).
+template <typename Real, class LAT, bool Z3, class First>
+__device__ __forceinline__ void grad_coefficients(const MapArgs<Real>& a, int cell, const double* basis, double ur,
+                                                  First&& draw_first, double& mine, double& rho_out,
+                                                  uint32_t& nnew) {
     constexpr int Q = LAT::Q;
     constexpr int NM = LAT::ORDER >= 3 ? kMoments : 10;  // raw moments of the order
     constexpr int W = kL2DWarps;
@@ -421,11 +450,12 @@ __device__ __forceinline__ void grad_coefficients(const MapArgs<Real>& a, int ce
     const int ix = cell % a.ncx, iy = (cell / a.ncx) % a.ncy, iz = cell / (a.ncx * a.ncy);
     constexpr int KN = Z3 ? 8 : 4;  // lb_ratio <= 2
     const int nk = Z3 ? r * r * r : r * r;
+    Real p[KN];
+#pragma unroll
+    for (int k = 0; k < KN; ++k) p[k] = 0;
     if (t < Q) {
-        Real p[KN];
 #pragma unroll
         for (int k = 0; k < KN; ++k) {
-            p[k] = 0;
             if (k < nk) {
                 const int dz = Z3 ? k / (r * r) : 0, dy = (k / r) % r, dx = k % r;
                 const int64_t node =
@@ -433,6 +463,9 @@ __device__ __forceinline__ void grad_coefficients(const MapArgs<Real>& a, int ce
                 p[k] = a.f[(int64_t)t * a.nnodes + node];
             }
         }
+    }
+    draw_first();
+    if (t < Q) {
         double sum = 0.0;
 #pragma unroll
         for (int k = 0; k < KN; ++k)
@@ -442,40 +475,39 @@ __device__ __forceinline__ void grad_coefficients(const MapArgs<Real>& a, int ce
     }
     __syncthreads();
     if (lane < (unsigned)NM) {
-        const LatBasis<LAT>& B = lat_basis<LAT>();
         const int qa = w * QW, qb = qa + QW < Q ? qa + QW : Q;
         double part = 0.0;
-        for (int q = qa; q < qb; ++q) part = fma(s_f[q], B.b[q][lane], part);
+        for (int q = qa; q < qb; ++q) part = fma(s_f[q], basis[q * kMoments + lane], part);
         s_part[w][lane] = part;
     }
     __syncthreads();
     if (w != 0) return;
     double R = 0.0;
-    if (lane < (unsigned)NM)
-#pragma unroll
-        for (int v = 0; v < W; ++v) R += s_part[v][lane];
+    if (lane < (unsigned)NM) {  // (a tree: an FP64 addition has 66 cycles of latency)
+        static_assert(W == 8, "the tree takes eight partials");
+        const double r0 = s_part[0][lane] + s_part[1][lane], r1 = s_part[2][lane] + s_part[3][lane];
+        const double r2 = s_part[4][lane] + s_part[5][lane], r3 = s_part[6][lane] + s_part[7][lane];
+        R = (r0 + r1) + (r2 + r3);
+    }
     auto at = [&](int k) { return __shfl_sync(kFull, R, k); };
     const double rho = at(0);
+    const double ne = floor(rho * (double)a.ppc + ur);
+    nnew = ne > 0.0 ? (uint32_t)ne : 0u;
     double inv = 0.0;
     if (lane == 0) inv = 1.0 / rho;  // one FP64 reciprocal, broadcast
     inv = __shfl_sync(kFull, inv, 0);
-    const double u[3] = {at(1) * inv, at(2) * inv, at(3) * inv};
-    double R2[6];
-#pragma unroll
-    for (int k = 0; k < 6; ++k) R2[k] = at(4 + k);
+    // the indices of the lane's coefficient (lanes 4-9 a2, 10-19 a3) and what it takes of the others,
+    // fetched by shuffles (tables indexed by the lane would sit in local memory)
+    int ci, cj, ck;
+    packed_indices((int)lane, ci, cj, ck);
+    const double ui = at(1 + ci) * inv, uj = at(1 + cj) * inv, uk = at(1 + ck) * inv;
+    const double Rjk = at(4 + packed_pair_index(cj, ck)), Rik = at(4 + packed_pair_index(ci, ck)),
+                 Rij = at(4 + packed_pair_index(ci, cj));
     double val = 0.0;
-    if (lane >= 4u && lane < 10u) {
-        int i, j;
-        packed_pair((int)lane - 4, i, j);
-        val = R * inv - u[i] * u[j] - (i == j ? 1.0 : 0.0);
-    } else if (lane >= 10u && lane < (unsigned)NM) {
-        constexpr int T[10][3] = {{0, 0, 0}, {0, 0, 1}, {0, 0, 2}, {0, 1, 1}, {0, 1, 2},
-                                  {0, 2, 2}, {1, 1, 1}, {1, 1, 2}, {1, 2, 2}, {2, 2, 2}};
-        const int i = T[lane - 10u][0], j = T[lane - 10u][1], k = T[lane - 10u][2];
-        const double cross = u[i] * R2[packed_pair_index(j, k)] + u[j] * R2[packed_pair_index(i, k)] +
-                             u[k] * R2[packed_pair_index(i, j)];
-        val = (R - cross) * inv + 2.0 * u[i] * u[j] * u[k];
-    }
+    if (lane >= 4u && lane < 10u)
+        val = R * inv - ui * uj - (ci == cj ? 1.0 : 0.0);
+    else if (lane >= 10u && lane < (unsigned)NM)
+        val = (R - (ui * Rjk + uj * Rik + uk * Rij)) * inv + 2.0 * ui * uj * uk;
     // M = max |val| over the lanes: the bits of non-negative doubles order as unsigned integers
     // (a NaN coefficient is left out, as fmax does)
     unsigned long long mb = val == val ? (unsigned long long)__double_as_longlong(fabs(val)) : 0ull;
@@ -489,9 +521,8 @@ __device__ __forceinline__ void grad_coefficients(const MapArgs<Real>& a, int ce
     // 16-18 u, lane 19 C
     const double mv = __shfl_sync(kFull, val, (int)(lane + 4u) & 31);
     mine = lane < (unsigned)(NM - 4) ? mv : 0.0;
-    if (lane == GR_U) mine = u[0];
-    if (lane == GR_U + 1) mine = u[1];
-    if (lane == GR_U + 2) mine = u[2];
+    const double us = at(1 + ((int)lane - GR_U) % 3) * inv;
+    if (lane >= (unsigned)GR_U && lane < (unsigned)(GR_U + 3)) mine = us;
     if (lane == GR_C) mine = 1.0 + 30.0 * M;
     rho_out = rho;
 }
@@ -524,7 +555,7 @@ __device__ __forceinline__ MoveCtx<Real> l2d_move_ctx(const MapArgs<Real>& a) {
 }
 
 template <typename Real, class LAT, bool Z3, bool MOVE = false>
-__device__ __forceinline__ void l2d_cells(const MapArgs<Real>& a, int first, int stride) {
+__device__ __forceinline__ void l2d_cells(const MapArgs<Real>& a, int first, int stride, const double* basis) {
     __shared__ unsigned s_am[kL2DWarps], s_em[kL2DWarps], s_vm[kL2DWarps];
     __shared__ Real s_c[20];
     __shared__ uint32_t s_nnew;
@@ -548,8 +579,22 @@ __device__ __forceinline__ void l2d_cells(const MapArgs<Real>& a, int first, int
         // the channel's cell: the key of the cell's random streams and of the stable order
         const uint32_t gcell = global_cell(cell, a.ncx, a.ncy, a.y0, a.ncy_g);
         const uint32_t old = threadIdx.x == 0 ? a.count[cell] : 0u;
+        // the draws of a trial: the unit Maxwellian (X, Y, Z) and the words of R and the position
+        Real X = 0, Y = 0, Z = 0;
+        uint4 r2 = make_uint4(0u, 0u, 0u, 0u);
+        auto draw_trial = [&](uint32_t j) {
+            const uint4 r1 = draw(a.seed, gcell, t_step, TAG_L2D_VEL, j, 0);
+            r2 = draw(a.seed, gcell, t_step, TAG_L2D_VEL, j, 1);
+            Real spare;
+            gauss_pair<Real>(r1.x, r1.y, X, Y);
+            gauss_pair<Real>(r1.z, r1.w, Z, spare);
+        };
         double mine = 0.0, rho = 0.0;
-        grad_coefficients<Real, LAT, Z3>(a, icell, mine, rho);  // the block; results in warp 0
+        uint32_t new_count = 0;
+        const double ur = w == 0 ? u01d(draw(a.seed, gcell, t_step, TAG_L2D_ROUND, 0, 0).x) : 0.0;
+        // the block; results in warp 0. The first trials are drawn while the populations come in
+        grad_coefficients<Real, LAT, Z3>(a, icell, basis, ur, [&]() { draw_trial(threadIdx.x); }, mine, rho,
+                                         new_count);
         if (w == 0) {
             GradRec& g = a.grad[ci];
             if (lane < 20u) {
@@ -557,12 +602,9 @@ __device__ __forceinline__ void l2d_cells(const MapArgs<Real>& a, int first, int
                 g.v[lane] = mine;
             }
             if (lane == 0) {
-                const double ur = u01d(draw(a.seed, gcell, t_step, TAG_L2D_ROUND, 0, 0).x);
-                const double ne = floor(rho * (double)a.ppc + ur);
-                const uint32_t nnew = ne > 0.0 ? (uint32_t)ne : 0u;
-                s_nnew = nnew;
+                s_nnew = new_count;
                 g.rho = rho;
-                g.nnew = nnew;
+                g.nnew = new_count;
                 g.pad = 0;
             }
         }
@@ -618,14 +660,8 @@ __device__ __forceinline__ void l2d_cells(const MapArgs<Real>& a, int first, int
             const uint32_t j = j0 + threadIdx.x;
             const bool valid = j < cap;
             bool acc = false, env = false;
-            Real X = 0, Y = 0, Z = 0;
-            uint4 r2 = make_uint4(0u, 0u, 0u, 0u);
             if (valid) {
-                const uint4 r1 = draw(a.seed, gcell, t_step, TAG_L2D_VEL, j, 0);
-                r2 = draw(a.seed, gcell, t_step, TAG_L2D_VEL, j, 1);
-                Real spare;
-                gauss_pair<Real>(r1.x, r1.y, X, Y);
-                gauss_pair<Real>(r1.z, r1.w, Z, spare);
+                if (j0 > 0) draw_trial(j);
                 const Real G = grad_G<Real, LAT::ORDER>(a2, a3, X, Y, Z);
                 const Real R = (Real)u01f(r2.x);
                 env = G > C;
@@ -739,16 +775,25 @@ __device__ __forceinline__ void l2d_cells(const MapArgs<Real>& a, int first, int
     if (lane == 0 && flags) atomicOr(&a.ctrl[CTRL_STATUS], flags);
 }
 
-// LB2DSMC: one block per listed cell (the listed cells of all replicas in the batch form).
-template <typename Real, class LAT, bool BATCH, bool Z3 = false, bool MOVE = false>
-__global__ void __launch_bounds__(kL2DWarps * 32) k_l2d(Launch<MapArgs<Real>> L) {
+// LB2DSMC: one block per listed cell (the listed cells of all replicas in the batch form). MB: blocks
+// an SM is to hold. Long lists are bound by how many cells an SM has in its FP64 solve at once:
+// 4 blocks in FP32 (2048 cells in 3D, 20 hybrid steps: 8.43 ms, with 3 or 2 blocks 8.51 or
+// 8.80 ms); lists of up to two cells per SM by one cell's latency: 2 blocks, which keep the
+// registers (256 cells, 20 steps: 1.254 ms, with 3 or 4 blocks 1.269 or 1.287 ms).
+template <typename Real, class LAT, bool BATCH, bool Z3 = false, bool MOVE = false, int MB = 2>
+__global__ void __launch_bounds__(kL2DWarps * 32, sizeof(Real) == 4 ? MB : 1) k_l2d(Launch<MapArgs<Real>> L) {
+    // the basis does not depend on the previous kernel: it is fetched while that one finishes
+    __shared__ double s_basis[LAT::Q * kMoments];
+    for (int i = threadIdx.x; i < LAT::Q * kMoments; i += kL2DWarps * 32)
+        s_basis[i] = lat_basis<LAT>().b[i / kMoments][i % kMoments];
     pdl_begin();
+    __syncthreads();
     if constexpr (BATCH) {
         const int r = replica_of(L.pre, L.nrep, (int64_t)blockIdx.x);
         const MapArgs<Real>& a = L.tab[r];
-        l2d_cells<Real, LAT, Z3, MOVE>(a, (int)(blockIdx.x - L.pre[r]), a.n);
+        l2d_cells<Real, LAT, Z3, MOVE>(a, (int)(blockIdx.x - L.pre[r]), a.n, s_basis);
     } else {
-        l2d_cells<Real, LAT, Z3, MOVE>(L.one, (int)blockIdx.x, (int)gridDim.x);
+        l2d_cells<Real, LAT, Z3, MOVE>(L.one, (int)blockIdx.x, (int)gridDim.x, s_basis);
     }
 }
 
@@ -795,29 +840,36 @@ cudaError_t d2l_impl(Ctx& c, const int32_t* nodes, int32_t n) {
     Launch<MapArgs<Real>> L{};
     L.one = a;
     L.total = n;
-    const cudaError_t e = launch_pdl(k_d2l<Real, LAT, false>, dim3(blocks_for(c, (int64_t)n * 32, 128, 16)),
+    const cudaError_t e = launch_pdl(k_d2l<Real, LAT, false>,
+                                     dim3(blocks_for(c, ((int64_t)n + a.lb_ratio - 1) / a.lb_ratio * 32, 128, 16)),
                                      dim3(128), 0, c.stream, L);
     prof_end(c, K_D2L);
     return e;
 }
 
-template <typename Real, class LAT>
+template <typename Real, class LAT, bool MOVE>
 cudaError_t l2d_launch(Ctx& c, const MapArgs<Real>& a, int32_t n) {
     prof_begin(c, K_L2D);
     Launch<MapArgs<Real>> L{};
     L.one = a;
     L.total = n;
-    const dim3 grid(blocks_for(c, (int64_t)n * 32 * kL2DWarps, 32 * kL2DWarps, 8));
-    const cudaError_t e =
-        a.ncz ? launch_pdl(k_l2d<Real, LAT, false, true>, grid, dim3(32 * kL2DWarps), 0, c.stream, L)
-              : launch_pdl(k_l2d<Real, LAT, false, false>, grid, dim3(32 * kL2DWarps), 0, c.stream, L);
+    const dim3 grid(blocks_for(c, (int64_t)n * 32 * kL2DWarps, 32 * kL2DWarps, 8)), block(32 * kL2DWarps);
+    constexpr int LONG = sizeof(Real) == 4 ? 4 : 2;  // (in FP64 the same kernel)
+    const bool longer = n > 2 * c.num_sms;
+    cudaError_t e;
+    if (a.ncz)
+        e = longer ? launch_pdl(k_l2d<Real, LAT, false, true, MOVE, LONG>, grid, block, 0, c.stream, L)
+                   : launch_pdl(k_l2d<Real, LAT, false, true, MOVE>, grid, block, 0, c.stream, L);
+    else
+        e = longer ? launch_pdl(k_l2d<Real, LAT, false, false, MOVE, LONG>, grid, block, 0, c.stream, L)
+                   : launch_pdl(k_l2d<Real, LAT, false, false, MOVE>, grid, block, 0, c.stream, L);
     prof_end(c, K_L2D);
     return e;
 }
 
 template <typename Real, class LAT>
 cudaError_t l2d_impl(Ctx& c, const int32_t* cells, int32_t n) {
-    return l2d_launch<Real, LAT>(c, map_args<Real>(c, cells, n), n);
+    return l2d_launch<Real, LAT, false>(c, map_args<Real>(c, cells, n), n);
 }
 
 // LB2DSMC of the fused pass of parity p: the listed cells' particles are in half p^1, the
@@ -832,16 +884,7 @@ cudaError_t l2d_move_impl(Ctx& c, const int32_t* cells, int32_t n, int p) {
     a.acount = c.st.count[p];
     a.dt_r = (Real)c.d.dt;
     a.g_r = (Real)c.d.g_step;
-    prof_begin(c, K_L2D);
-    Launch<MapArgs<Real>> L{};
-    L.one = a;
-    L.total = n;
-    const dim3 grid(blocks_for(c, (int64_t)n * 32 * kL2DWarps, 32 * kL2DWarps, 8));
-    const cudaError_t e =
-        a.ncz ? launch_pdl(k_l2d<Real, LAT, false, true, true>, grid, dim3(32 * kL2DWarps), 0, c.stream, L)
-              : launch_pdl(k_l2d<Real, LAT, false, false, true>, grid, dim3(32 * kL2DWarps), 0, c.stream, L);
-    prof_end(c, K_L2D);
-    return e;
+    return l2d_launch<Real, LAT, true>(c, a, n);
 }
 
 constexpr int kMaxDevices = 64;
@@ -876,7 +919,7 @@ template <typename Real, class LAT>
 cudaError_t l2d_noalloc_impl(Ctx& c, const int32_t* cells, int32_t n, GradRec* rec) {
     MapArgs<Real> a = map_args<Real>(c, cells, n);
     a.grad = rec;  // the fixed array instead of the arena's records
-    return l2d_launch<Real, LAT>(c, a, n);
+    return l2d_launch<Real, LAT, false>(c, a, n);
 }
 
 }  // namespace
