@@ -140,6 +140,9 @@ struct LbmArgs {
     const Real* tau_node;
     int32_t bgk;  // 1: unregularised BGK collision (lb_collision)
     int32_t nz;   // lattice layers along z (1 in 2D)
+    // a batch's LB step ends its replicas' DSMC steps (end_of_step)
+    uint32_t* ctrl;
+    uint32_t sample_every;
 };
 
 // One step of the adjoint of the LBM with per-node parameters: lam_next = dL/df_{t+1} in,
@@ -166,6 +169,7 @@ struct MapArgs {
     int32_t nx, ny, ncx, ncy, lb_ratio, ppc, n, bin;
     int64_t nnodes;
     const int32_t* list;
+    uint32_t pending;  // a batch's DSMC2LB, whose DSMC step is not ended yet: sample_every; else 0
     int32_t eq_mode;  // DSMC2LB: 1 the local equilibrium of rho, u only (d2l_mode)
     double r_lat;
     uint64_t seed;
@@ -246,16 +250,29 @@ struct Launch {
     int64_t total;        // units of the launch
 };
 
+// Called by a whole warp for one unit: the lanes read 32 offsets of the range at a time, two
+// dependent loads for up to 1024 replicas (a bisection by each thread took six for 64 replicas,
+// on the path of every block of every kernel).
 __device__ __forceinline__ int replica_of(const int64_t* pre, int nrep, int64_t u) {
+    const int lane = (int)(threadIdx.x & 31u);
     int lo = 0, hi = nrep;
     while (hi - lo > 1) {
-        const int mid = (lo + hi) >> 1;
-        if (pre[mid] <= u)
-            lo = mid;
-        else
-            hi = mid;
+        const int step = (hi - lo + 31) / 32;
+        const int i = lo + (lane + 1) * step;
+        lo += __popc(__ballot_sync(kFull, i < hi && pre[i] <= u)) * step;
+        hi = min(hi, lo + step);
     }
     return lo;
+}
+
+// The end of a DSMC step, once its collide pass is complete: the particles the pass counted
+// become the live count, and the step and sample counters advance.
+__device__ __forceinline__ void end_of_step(uint32_t* ctrl, uint32_t sample_every) {
+    const uint32_t s = ctrl[CTRL_STEP];
+    ctrl[CTRL_NTOT] = ctrl[CTRL_NACC];
+    ctrl[CTRL_NACC] = 0u;
+    if (sample_every == 1u || s % sample_every == 0u) ctrl[CTRL_NSAMPLES] += 1u;
+    ctrl[CTRL_STEP] = s + 1u;
 }
 
 // Programmatic dependent launch (sm_90 and later). The kernels of a step are launched with

@@ -305,11 +305,19 @@ template <typename Real, class LAT, bool BATCH, bool BGK = false, bool PARAM = f
 __global__ void __launch_bounds__(128) k_lbm(Launch<LbmArgs<Real>> L) {
     pdl_begin();
     const int64_t u = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (u >= L.total) return;
     if constexpr (BATCH) {
-        const int r = replica_of(L.pre, L.nrep, u);
+        if (blockIdx.x == gridDim.x - 1) {  // a block past the nodes ends the replicas' DSMC steps
+            for (int r = threadIdx.x; r < L.nrep; r += blockDim.x) end_of_step(L.tab[r].ctrl, L.tab[r].sample_every);
+            return;
+        }
+        const int64_t u0 = u - (int64_t)lane_id();  // the warp's first node
+        if (u0 >= L.total) return;
+        int r = replica_of(L.pre, L.nrep, u0);
+        if (u >= L.total) return;
+        while (u >= L.pre[r + 1]) ++r;
         lbm_node<Real, LAT, PARAM, BGK>(L.tab[r], u - L.pre[r]);
     } else {
+        if (u >= L.total) return;
         lbm_node<Real, LAT, PARAM, BGK, Z3>(L.one, u);
     }
 }
@@ -828,6 +836,8 @@ LbmArgs<Real> lbm_args(const Ctx& c, int cur_f) {
     a.tau_node = (const Real*)c.st.tau_node;  // Kn profile, or null
     a.bgk = c.p.lb_collision;
     a.nz = (int32_t)c.d.nz;
+    a.ctrl = c.st.ctrl;
+    a.sample_every = (uint32_t)c.p.sample_every;
     return a;
 }
 
@@ -951,7 +961,7 @@ cudaError_t batch_lbm_impl(BatchDev& b, int cur_f) {
     L.pre = b.pre_nodes;
     L.nrep = b.nrep;
     L.total = b.tot_nodes;
-    const int64_t blocks = (b.tot_nodes + b.lbm_block - 1) / b.lbm_block;
+    const int64_t blocks = (b.tot_nodes + b.lbm_block - 1) / b.lbm_block + 1;  // the last ends the DSMC steps
     if (b.lb_collision)
         return launch_pdl(k_lbm<Real, LAT, true, true>, dim3((unsigned)blocks), dim3(b.lbm_block), 0,
                           b.stream, L);

@@ -102,7 +102,9 @@ __device__ __forceinline__ void d2l_entries(const MapArgs<Real>& a, int first, i
     const Real* sx = lt.x;
     const Real* sw = lt.w;
     const unsigned lane = lane_id();
-    const uint32_t S = a.ctrl[CTRL_NSAMPLES];
+    uint32_t S = a.ctrl[CTRL_NSAMPLES];
+    // the sample of a step that a batch's LB step is still to end
+    if (a.pending && (a.pending == 1u || a.ctrl[CTRL_STEP] % a.pending == 0u)) S += 1u;
     constexpr int NH = (LAT::Q + 31) / 32;
     for (int t0 = first * per; t0 < a.n; t0 += stride * per) {
         int64_t have = -1;  // the cell whose populations f holds
@@ -1017,10 +1019,12 @@ void map_args_fill(Ctx& c, int cur_p, int cur_f, const int32_t* list, int32_t n,
     c.cur_p = cur_p;
     c.cur_f = cur_f;
     if (c.p.real_bytes == 4) {
-        const MapArgs<float> a = map_args<float>(c, list, n);
+        MapArgs<float> a = map_args<float>(c, list, n);
+        a.pending = (uint32_t)c.p.sample_every;
         std::memcpy(out, &a, sizeof(a));
     } else {
-        const MapArgs<double> a = map_args<double>(c, list, n);
+        MapArgs<double> a = map_args<double>(c, list, n);
+        a.pending = (uint32_t)c.p.sample_every;
         std::memcpy(out, &a, sizeof(a));
     }
     c.cur_p = sp;
