@@ -961,6 +961,7 @@ def _lb_forward(h, g, tau, f0, nsteps, ckpt_every):
 def _loss_forward(h, g, tau, f0, nodes, targets, nsteps, ckpt_every):
     """Loss after nsteps LB steps from f0, dL/df_T, and the checkpoints of the states."""
     torch = h.torch
+    h.stream.wait_stream(torch.cuda.current_stream(f0.device))  # the inputs may still be in the making
     with torch.cuda.stream(h.stream):
         fT, ckpts = _lb_forward(h, g, tau, f0, nsteps, ckpt_every)
         loss = torch.zeros(1, dtype=torch.float64, device=f0.device)
