@@ -624,11 +624,13 @@ __device__ __forceinline__ void adjoint_wall_row(const LbmAdjArgs<Real>& a, int 
 }
 
 // One thread per node: the collision adjoint and the transposed pull. A row is cut into segments
-// of equal width, at most 32 nodes, a warp each, so that the nodes next to a wall (as many as the
-// largest speed, three at most, and a row has at least six) are in one warp, which adds up the
-// row's wall adjoint and writes the populations it feeds. Bound by latency at 256 x 128 nodes (1.7
-// warps per scheduler). There the last block of a grid-wide ticket, which spread the sums of every
-// row, ran alone for half of the kernel's time: a gradient of 100 steps took 3.58 ms, of which the
+// of at most 32 nodes, a warp each, that differ by at most one node: a row of more than 32 nodes has at
+// least 16 in each, a shorter one is a single segment (of six nodes or more), so the nodes next to a
+// wall (as many as the largest speed, three at most) are always in one warp, which adds up the
+// row's wall adjoint and writes the populations it feeds. (Segments of one width with a remainder left
+// one or two nodes in the last one at 962, 993, 994, 1025 nodes and on.) Bound by latency at 256 x 128
+// nodes (1.7 warps per scheduler). There the last block of a grid-wide ticket, which spread the sums of
+// every row, ran alone for half of the kernel's time: a gradient of 100 steps took 3.58 ms, of which the
 // adjoint 24.7 us a step; without the tail and with the launches overlapped 2.09 ms.
 // With `early` the populations at t are known to be complete when the previous kernel of the
 // stream starts its work, and the forward moments are formed before that kernel has finished: the
@@ -636,12 +638,14 @@ __device__ __forceinline__ void adjoint_wall_row(const LbmAdjArgs<Real>& a, int 
 // wait), so at most the previous kernel is still running then.
 template <typename Real, class LAT, bool Z3 = false>
 __global__ void __launch_bounds__(128) k_lbm_adj(LbmAdjArgs<Real> a) {
+    static_assert(LAT::MAXV <= 6, "a segment holds the nodes next to a wall");
     const int wid = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5);
     const int row = wid / a.nseg, seg = wid - row * a.nseg;
     const unsigned lane = lane_id();
-    const int x0 = seg * a.width, x = x0 + (int)lane;
+    const int x0 = seg * a.width + min(seg, a.wider), width = a.width + (seg < a.wider ? 1 : 0);
+    const int x = x0 + (int)lane;
     const int y = Z3 ? row % a.ny : row, z = Z3 ? row / a.ny : 0;
-    const bool act = row < a.ny * a.nz && (int)lane < a.width && x < a.nx;
+    const bool act = row < a.ny * a.nz && (int)lane < width;
     NodeMoments<Real> nm;
     if (a.early && act) adjoint_moments<Real, LAT, Z3>(a, x, y, z, nm);
     pdl_after_wait();
@@ -653,7 +657,7 @@ __global__ void __launch_bounds__(128) k_lbm_adj(LbmAdjArgs<Real> a) {
     if (act) lbm_adjoint_node<Real, LAT, Z3>(a, x, y, z, nm, wl, wr);
     __syncwarp();
     if (x0 == 0 && lane == 0) adjoint_wall_row<Real, LAT, Z3, true>(a, y, z, wall_sum<LAT>(wl));
-    if (x0 + a.width >= a.nx && lane == 31) adjoint_wall_row<Real, LAT, Z3, false>(a, y, z, wall_sum<LAT>(wr));
+    if (x0 + width == a.nx && lane == 31) adjoint_wall_row<Real, LAT, Z3, false>(a, y, z, wall_sum<LAT>(wr));
 }
 
 // Packed index of the symmetric pair (i, j): xx xy xz yy yz zz.
@@ -921,7 +925,8 @@ cudaError_t lbm_adj_impl(Ctx& c, const void* f, const void* lam_next, void* lam,
     a.nz = (int32_t)c.d.nz;
     a.nnodes = c.d.nnodes;
     a.nseg = (a.nx + 31) / 32;
-    a.width = (a.nx + a.nseg - 1) / a.nseg;
+    a.width = a.nx / a.nseg;
+    a.wider = a.nx % a.nseg;
     a.early = early ? 1 : 0;
     const int64_t warps = (int64_t)a.nseg * a.ny * a.nz;
     const dim3 grid((unsigned)((warps + 3) / 4)), b(128);  // (32 or 64 threads: 8% or 2% slower)
