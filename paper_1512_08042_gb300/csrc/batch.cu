@@ -232,6 +232,7 @@ hyb_status hyb_batch_init(const hyb_params* p, int32_t n, void* arena, uint64_t 
     d.lb_collision = p[0].lb_collision;
     d.stream = b->stream;
     d.num_sms = b->reps[0]->c.num_sms;
+    d.smem_block = b->reps[0]->c.smem_block;
     b->cur_p = b->reps[0]->c.cur_p;
     b->cur_f = b->reps[0]->c.cur_f;
     b->tab = b->arena + off[n];

@@ -571,6 +571,7 @@ struct BatchDev {
     int32_t real_bytes = 4, lattice = 39;
     int32_t lb_collision = 0;  // one collision for all replicas
     int num_sms = 152;
+    int smem_block = 232448;  // shared memory a block may have, bytes
     cudaStream_t stream = nullptr;
     const void* dsmc[2] = {nullptr, nullptr};               // DsmcArgs<Real>[nrep], by particle half
     const void* lbm[2] = {nullptr, nullptr};                // LbmArgs<Real>[nrep], by population half
@@ -624,6 +625,7 @@ struct Ctx {
     int cur_f = 0;  // current population half
     State st{};
     int num_sms = 152;
+    int smem_block = 232448;  // shared memory a block may have, bytes
     std::string err;
     // kernel timing
     int prof_kernel = -1;

@@ -283,6 +283,7 @@ struct CollideCfg {
     static constexpr int MINB = (sizeof(Real) == 4 ? 24 : 16) / W;  // resident blocks per SM
 };
 enum CollideMode : int { MODE_COLLIDE = 0, MODE_FUSED = 1 };
+constexpr int kCollideStatic = 64;  // bytes, at least the block's event sums beside the warps' memory
 
 // Words of a cell's order-key bitmap: one bit per key below W bin, W = 9 neighbour offsets in
 // 2D and 27 in 3D (bin is a multiple of 32).
@@ -892,6 +893,7 @@ __global__ void __launch_bounds__(W * 32, (CollideCfg<Real, W>::MINB))
     k_collide(Launch<DsmcArgs<Real>> L, uint32_t pool, uint32_t warp_smem) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ uint32_t s_tot[4], s_done;
+    static_assert(sizeof(s_tot) + sizeof(s_done) <= kCollideStatic, "fitting_pool counts them");
     if (threadIdx.x < 4) s_tot[threadIdx.x] = 0u;
     if (threadIdx.x == 4) s_done = 0u;
     __syncthreads();
@@ -1098,6 +1100,19 @@ cudaError_t move_impl(Ctx& c, int p) {
     return e;
 }
 
+// Pool slots of a collide warp in a block of `warps`: as many of the wanted `pool` (collide_pool) as
+// leave the block within the shared memory a block may have (limit), and at least one bin, which the
+// largest bins leave room for in either shape. A smaller pool only has more warps take their cells one
+// at a time. Bins of 128 to 256 slots need it: in blocks of 8 warps from 95 particles per cell on in
+// FP64 3D (at a capacity factor of 2.5), 132 in FP64 2D and 189 in FP32 3D, in blocks of 4 from 223 in
+// FP64 3D.
+template <typename Real, bool Z3>
+uint32_t fitting_pool(uint32_t pool, uint32_t bin, int warps, int limit) {
+    const uint32_t per_warp = (uint32_t)((limit - kCollideStatic) / warps);
+    while (pool > bin && warp_mem<Real, Z3>(pool, bin).total > per_warp) pool -= 8u;
+    return pool;
+}
+
 template <typename Real, bool Z3, int MODE, int W>
 cudaError_t collide_impl_w(Ctx& c, int p) {
     const int save = c.cur_p;
@@ -1106,7 +1121,7 @@ cudaError_t collide_impl_w(Ctx& c, int p) {
     L.one = make_args<Real>(c);
     c.cur_p = save;
     constexpr int NC = W * kWarpCells;
-    const uint32_t pool = collide_pool(c);
+    const uint32_t pool = fitting_pool<Real, Z3>(collide_pool(c), (uint32_t)c.d.bin, W, c.smem_block);
     const uint32_t warp_smem = warp_mem<Real, Z3>(pool, (uint32_t)c.d.bin).total;
     const size_t smem = (size_t)W * warp_smem;
     // (dynamic and static shared memory together may exceed the default 48 KB)
@@ -1239,23 +1254,19 @@ int collide_per_sm(Kern kernel, int threads, size_t smem) {
 // slowest block, which the fused pass lengthens (a collide and a move in one block), and two
 // separate passes are faster.
 namespace {
+template <typename Real, bool Z3, int W>
+int fused_per_sm(const Ctx& c) {
+    const uint32_t bin = (uint32_t)c.d.bin;
+    const uint32_t pool = fitting_pool<Real, Z3>(collide_pool(c), bin, W, c.smem_block);
+    return collide_per_sm(k_collide<Real, false, Z3, MODE_FUSED, W>, W * 32,
+                          (size_t)W * warp_mem<Real, Z3>(pool, bin).total);
+}
 template <int W>
 bool fused_fills_gpu_w(const Ctx& c) {
     constexpr int NC = W * kWarpCells;
-    const uint32_t pool = collide_pool(c);
-    const uint32_t bin = (uint32_t)c.d.bin;
     const bool z3 = c.p.ncz >= 2;
-    int per_sm;
-    if (c.p.real_bytes == 4)
-        per_sm = z3 ? collide_per_sm(k_collide<float, false, true, MODE_FUSED, W>, W * 32,
-                                     (size_t)W * warp_mem<float, true>(pool, bin).total)
-                    : collide_per_sm(k_collide<float, false, false, MODE_FUSED, W>, W * 32,
-                                     (size_t)W * warp_mem<float, false>(pool, bin).total);
-    else
-        per_sm = z3 ? collide_per_sm(k_collide<double, false, true, MODE_FUSED, W>, W * 32,
-                                     (size_t)W * warp_mem<double, true>(pool, bin).total)
-                    : collide_per_sm(k_collide<double, false, false, MODE_FUSED, W>, W * 32,
-                                     (size_t)W * warp_mem<double, false>(pool, bin).total);
+    const int per_sm = c.p.real_bytes == 4 ? (z3 ? fused_per_sm<float, true, W>(c) : fused_per_sm<float, false, W>(c))
+                                           : (z3 ? fused_per_sm<double, true, W>(c) : fused_per_sm<double, false, W>(c));
     if (per_sm < 1) return true;
     const int64_t blocks = (c.d.ncells + NC - 1) / NC;
     return blocks >= (int64_t)per_sm * c.num_sms;
@@ -1266,9 +1277,9 @@ bool dsmc_fused_fills_gpu(const Ctx& c) {
     return c.collide_warps == 4 ? fused_fills_gpu_w<4>(c) : fused_fills_gpu_w<8>(c);
 }
 
-// Pool slots of a collide warp: its four cells' counts add up to about 4 ppc with a spread of
+// Pool slots a collide warp should have: its four cells' counts add up to about 4 ppc with a spread of
 // sqrt(4 ppc); room for four such spreads (a warp whose cells do not fit takes the pool one
-// cell at a time), and at least one full bin.
+// cell at a time), and at least one full bin (what a block has room for: fitting_pool).
 uint32_t collide_pool(const Ctx& c) {
     const double mean = (double)kWarpCells * c.p.ppc;
     uint32_t pool = ((uint32_t)std::ceil(mean + 4.0 * std::sqrt(mean)) + 7u) / 8u * 8u;
@@ -1296,20 +1307,22 @@ cudaError_t batch_collide_impl(BatchDev& b, int cur_p) {
     L.tab = (const DsmcArgs<Real>*)b.dsmc[cur_p];
     L.nrep = b.nrep;
     cudaError_t e;
-    const uint32_t warp_smem = warp_mem<Real, false>(b.pool, b.maxbin).total;
-    const size_t smem = (size_t)(b.collide_block / 32) * warp_smem;
+    const int warps = b.collide_block / 32;
+    const uint32_t pool = fitting_pool<Real, false>(b.pool, b.maxbin, warps, b.smem_block);
+    const uint32_t warp_smem = warp_mem<Real, false>(pool, b.maxbin).total;
+    const size_t smem = (size_t)warps * warp_smem;
     if (b.collide_block == 128) {  // blocks of 16 cells
         L.pre = b.pre_blocks4;
         L.total = b.tot_blocks4;
         auto k = k_collide<Real, true, false, MODE_COLLIDE, 4>;
         e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e == cudaSuccess) e = launch_pdl(k, dim3((unsigned)L.total), dim3(128), smem, b.stream, L, b.pool, warp_smem);
+        if (e == cudaSuccess) e = launch_pdl(k, dim3((unsigned)L.total), dim3(128), smem, b.stream, L, pool, warp_smem);
     } else {  // blocks of 32 cells
         L.pre = b.pre_blocks;
         L.total = b.tot_blocks;
         auto k = k_collide<Real, true, false, MODE_COLLIDE, 8>;
         e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e == cudaSuccess) e = launch_pdl(k, dim3((unsigned)L.total), dim3(256), smem, b.stream, L, b.pool, warp_smem);
+        if (e == cudaSuccess) e = launch_pdl(k, dim3((unsigned)L.total), dim3(256), smem, b.stream, L, pool, warp_smem);
     }
     return e;  // (the batch's LB step ends the DSMC step)
 }

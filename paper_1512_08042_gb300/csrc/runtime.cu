@@ -477,6 +477,7 @@ hyb_status dsmc_init(const hyb_params* p, void* arena, uint64_t arena_bytes, voi
     resolve(c);
     cudaGetDevice(&c.device);
     cudaDeviceGetAttribute(&c.num_sms, cudaDevAttrMultiProcessorCount, c.device);
+    cudaDeviceGetAttribute(&c.smem_block, cudaDevAttrMaxSharedMemoryPerBlockOptin, c.device);
     // pinned host words for status reads, followed by the timing pool
     void* hp = nullptr;
     if (cudaMallocHost(&hp, 256) != cudaSuccess) {
