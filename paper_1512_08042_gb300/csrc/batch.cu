@@ -432,6 +432,8 @@ hyb_status hyb_batch_tune(hyb_batch* b, const int32_t* dev_nodes, const int64_t*
     // DSMC2LB
     hyb_status s = HYB_OK;
     const int order[4] = {hyb::K_MOVE, hyb::K_COLLIDE, hyb::K_LBM, hyb::K_D2L};
+    int before[4];
+    for (int ki = 0; ki < 4; ++ki) before[ki] = hyb_batch_get_block(b, order[ki]);
     for (int ki = 0; ki < 4 && s == HYB_OK; ++ki) {
         const int k = order[ki];
         int best_t = hyb_batch_get_block(b, k);
@@ -449,7 +451,10 @@ hyb_status hyb_batch_tune(hyb_batch* b, const int32_t* dev_nodes, const int64_t*
     }
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
-    if (s != HYB_OK) return s;
+    if (s != HYB_OK) {  // the batch keeps what it had
+        for (int ki = 0; ki < 4; ++ki) hyb_batch_set_block(b, order[ki], before[ki]);
+        return s;
+    }
     if (move_block) *move_block = b->dev.move_block;
     if (lbm_block) *lbm_block = b->dev.lbm_block;
     return s;

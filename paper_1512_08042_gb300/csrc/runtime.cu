@@ -786,6 +786,7 @@ hyb_status hyb_tune_collide(hyb_ctx* h, const int32_t* dev_nodes, int32_t n_node
     constexpr int kSteps = 8, kReplays = 4;
     const int shapes[4] = {8, 4, 8, 4};
     const int modes[4] = {HYB_FUSE_ALWAYS, HYB_FUSE_ALWAYS, HYB_FUSE_NEVER, HYB_FUSE_NEVER};
+    const int warps_before = c.collide_warps, mode_before = c.fuse_mode;
     float best = 1e30f;
     int best_i = 0;
     hyb_status s = HYB_OK;
@@ -811,7 +812,11 @@ hyb_status hyb_tune_collide(hyb_ctx* h, const int32_t* dev_nodes, int32_t n_node
     }
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
-    if (s != HYB_OK) return s;
+    if (s != HYB_OK) {  // the context keeps what it had
+        hyb_set_collide_block(h, warps_before);
+        hyb_set_fuse(h, mode_before);
+        return s;
+    }
     s = hyb_set_collide_block(h, shapes[best_i]);
     if (s == HYB_OK) s = hyb_set_fuse(h, modes[best_i]);
     if (warps) *warps = shapes[best_i];
