@@ -149,7 +149,7 @@ struct LbmArgs {
 // lam = dL/df_t out, the parameter gradients accumulated. A row of nx nodes is cut into nseg
 // segments, a warp each: the first `wider` of width + 1 nodes, the others of `width` (at most 32
 // nodes each). early: the populations at t were complete before the previous kernel of the stream
-// began its work.
+// began its work. ahead: the next kernel's blocks may be placed while this one runs.
 template <typename Real>
 struct LbmAdjArgs {
     const Real* f;         // populations at t
@@ -160,7 +160,7 @@ struct LbmAdjArgs {
     Real* grad_g;
     Real* grad_tau;
     int32_t nx, ny, nz;
-    int32_t nseg, width, wider, early;
+    int32_t nseg, width, wider, early, ahead;
     int64_t nnodes;
 };
 
@@ -287,10 +287,11 @@ __device__ __forceinline__ void pdl_begin() {
 }
 
 // For kernels whose next one may read, before its own wait, what was complete before this kernel
-// began its work: the next kernel is scheduled only once this one's wait is over.
-__device__ __forceinline__ void pdl_after_wait() {
+// began its work: the next kernel is scheduled only once this one's wait is over. ahead = false: when
+// this one is over (a kernel without launch_dependents lets the next one start at its end).
+__device__ __forceinline__ void pdl_after_wait(bool ahead) {
     asm volatile("griddepcontrol.wait;" ::: "memory");
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    if (ahead) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
 
 // Asynchronous 16-byte copies from global to shared memory (cp.async, sm_80 and later),
