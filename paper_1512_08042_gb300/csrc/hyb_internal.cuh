@@ -146,10 +146,11 @@ struct LbmArgs {
 };
 
 // One step of the adjoint of the LBM with per-node parameters: lam_next = dL/df_{t+1} in,
-// lam = dL/df_t out, the parameter gradients accumulated. A row of nx nodes is cut into nseg
-// segments, a warp each: the first `wider` of width + 1 nodes, the others of `width` (at most 32
-// nodes each). early: the populations at t were complete before the previous kernel of the stream
-// began its work. ahead: the next kernel's blocks may be placed while this one runs.
+// lam = dL/df_t out, the parameter gradients accumulated. rows > 0: a block takes that many whole rows.
+// Otherwise a row of nx nodes is cut into nseg segments, a warp each: the first `wider` of width + 1
+// nodes, the others of `width` (at most 32 nodes each). early: the populations at t were complete
+// before the previous kernel of the stream began its work. ahead: the next kernel's blocks may be
+// placed while this one runs.
 template <typename Real>
 struct LbmAdjArgs {
     const Real* f;         // populations at t
@@ -160,7 +161,7 @@ struct LbmAdjArgs {
     Real* grad_g;
     Real* grad_tau;
     int32_t nx, ny, nz;
-    int32_t nseg, width, wider, early, ahead;
+    int32_t nseg, width, wider, rows, early, ahead;
     int64_t nnodes;
 };
 

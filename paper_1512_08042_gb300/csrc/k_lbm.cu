@@ -623,41 +623,69 @@ __device__ __forceinline__ void adjoint_wall_row(const LbmAdjArgs<Real>& a, int 
     });
 }
 
-// One thread per node: the collision adjoint and the transposed pull. A row is cut into segments
-// of at most 32 nodes, a warp each, that differ by at most one node: a row of more than 32 nodes has at
-// least 16 in each, a shorter one is a single segment (of six nodes or more), so the nodes next to a
-// wall (as many as the largest speed, three at most) are always in one warp, which adds up the
-// row's wall adjoint and writes the populations it feeds. (Segments of one width with a remainder left
-// one or two nodes in the last one at 962, 993, 994, 1025 nodes and on.) Bound by latency at 256 x 128
-// nodes (1.7 warps per scheduler). There the last block of a grid-wide ticket, which spread the sums of
-// every row, ran alone for half of the kernel's time: a gradient of 100 steps took 3.58 ms, of which the
-// adjoint 24.7 us a step; without the tail and with the launches overlapped 2.09 ms.
+// One thread per node: the collision adjoint and the transposed pull. The nodes next to a wall (as many
+// as the largest speed, three at most) add up their row's wall adjoint, and one of them writes the
+// populations it feeds. Two maps of nodes to threads:
+//   segments    a row is cut into segments of at most 32 nodes, a warp each, that differ by at most one
+//               node: a row of more than 32 nodes has at least 16 in each, a shorter one is a single
+//               segment (of six nodes or more), so the nodes next to a wall are always in one warp.
+//               (Segments of one width with a remainder left one or two nodes in the last one at 962,
+//               993, 994, 1025 nodes and on.)
+//   whole rows  a block takes as many whole rows as it has room for. Segments leave lanes empty on rows of
+//               less than a warp, and on rows a little wider: a block's four warps hold four rows of up
+//               to 32 nodes or two of up to 64, where the block has room for 21 rows of six nodes and
+//               three of up to 42. FP64, bound by the issue of its pipe, loses all of it (65k nodes,
+//               D3Q39, us a step, segments / whole rows: 6 nodes a row 781 / 180, 16 308 / 180, 33
+//               300 / 220); FP32 does on large lattices (524k nodes: 464 / 103, 180 / 102, 165 / 124).
+// Bound by latency at 256 x 128 nodes (1.7 warps per scheduler). There the last block of a grid-wide
+// ticket, which spread the sums of every row, ran alone for half of the kernel's time: a gradient of 100
+// steps took 3.58 ms, of which the adjoint 24.7 us a step; without the tail and with the launches
+// overlapped 2.09 ms.
 // With `early` the populations at t are known to be complete when the previous kernel of the
 // stream starts its work, and the forward moments are formed before that kernel has finished: the
 // next kernel may only be scheduled once this one's wait is over (launch_dependents after the
 // wait), so at most the previous kernel is still running then.
+constexpr int kAdjRows = 128 / 6;  // whole rows of a block at most (a row has at least six nodes)
 template <typename Real, class LAT, bool Z3 = false>
 __global__ void __launch_bounds__(128) k_lbm_adj(LbmAdjArgs<Real> a) {
-    static_assert(LAT::MAXV <= 6, "a segment holds the nodes next to a wall");
-    const int wid = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5);
-    const int row = wid / a.nseg, seg = wid - row * a.nseg;
+    static_assert(LAT::MAXV <= 6, "a row or a segment holds the nodes next to a wall");
+    const int nrows = a.ny * a.nz;
     const unsigned lane = lane_id();
-    const int x0 = seg * a.width + min(seg, a.wider), width = a.width + (seg < a.wider ? 1 : 0);
-    const int x = x0 + (int)lane;
+    int row, x, slot;       // the thread's node, and the wall sums it takes part in
+    bool act, first, last;  // first, last: the thread adds up the left, the right wall's sum
+    if (a.rows > 0) {
+        slot = (int)threadIdx.x / a.nx;
+        x = (int)threadIdx.x - slot * a.nx;
+        row = (int)blockIdx.x * a.rows + slot;
+        act = slot < a.rows && row < nrows;
+        first = act && x == 0;
+        last = act && x == a.nx - 1;
+    } else {
+        const int wid = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5);
+        row = wid / a.nseg;
+        const int seg = wid - row * a.nseg;
+        const int x0 = seg * a.width + min(seg, a.wider), width = a.width + (seg < a.wider ? 1 : 0);
+        x = x0 + (int)lane;
+        slot = (int)(threadIdx.x >> 5) & 3;
+        act = row < nrows && (int)lane < width;
+        first = row < nrows && x0 == 0 && lane == 0;
+        last = row < nrows && x0 + width == a.nx && lane == 31;
+    }
     const int y = Z3 ? row % a.ny : row, z = Z3 ? row / a.ny : 0;
-    const bool act = row < a.ny * a.nz && (int)lane < width;
     NodeMoments<Real> nm;
     if (a.early && act) adjoint_moments<Real, LAT, Z3>(a, x, y, z, nm);
     pdl_after_wait(sizeof(Real) == 4 || a.ahead);
-    if (row >= a.ny * a.nz) return;  // whole warps
     if (!a.early && act) adjoint_moments<Real, LAT, Z3>(a, x, y, z, nm);
-    __shared__ Real s_wall[4][2][wall_parts<LAT>()];
-    Real* wl = s_wall[(threadIdx.x >> 5) & 3][0];
-    Real* wr = s_wall[(threadIdx.x >> 5) & 3][1];
+    __shared__ Real s_wall[kAdjRows][2][wall_parts<LAT>()];
+    Real* wl = s_wall[min(slot, kAdjRows - 1)][0];
+    Real* wr = s_wall[min(slot, kAdjRows - 1)][1];
     if (act) lbm_adjoint_node<Real, LAT, Z3>(a, x, y, z, nm, wl, wr);
-    __syncwarp();
-    if (x0 == 0 && lane == 0) adjoint_wall_row<Real, LAT, Z3, true>(a, y, z, wall_sum<LAT>(wl));
-    if (x0 + width == a.nx && lane == 31) adjoint_wall_row<Real, LAT, Z3, false>(a, y, z, wall_sum<LAT>(wr));
+    if (a.rows > 0)
+        __syncthreads();
+    else
+        __syncwarp();
+    if (first) adjoint_wall_row<Real, LAT, Z3, true>(a, y, z, wall_sum<LAT>(wl));
+    if (last) adjoint_wall_row<Real, LAT, Z3, false>(a, y, z, wall_sum<LAT>(wr));
 }
 
 // Packed index of the symmetric pair (i, j): xx xy xz yy yz zz.
@@ -940,8 +968,14 @@ cudaError_t lbm_adj_impl(Ctx& c, const void* f, const void* lam_next, void* lam,
     a.width = a.nx / a.nseg;
     a.wider = a.nx % a.nseg;
     a.early = early ? 1 : 0;
-    const int64_t warps = (int64_t)a.nseg * a.ny * a.nz;
-    const dim3 grid((unsigned)((warps + 3) / 4)), b(128);  // (32 or 64 threads: 8% or 2% slower)
+    const int64_t nrows = (int64_t)a.ny * a.nz, warps = a.nseg * nrows;
+    // whole rows where a block then holds more of them than its four warps' segments do; rows of more
+    // than one segment only on lattices of more than two warps per scheduler, below which the kernel is
+    // bound by latency and the segments, without a block barrier, are 2% faster
+    const int whole = 128 / a.nx;
+    a.rows = whole * a.nseg > 4 && (a.nseg == 1 || warps > 8 * (int64_t)c.num_sms) ? whole : 0;
+    const int64_t blocks = a.rows > 0 ? (nrows + a.rows - 1) / a.rows : (warps + 3) / 4;
+    const dim3 grid((unsigned)blocks), b(128);  // (32 or 64 threads: 8% or 2% slower)
     a.ahead = next_ahead<Real>(c, grid.x) ? 1 : 0;
     return a.nz > 1 ? launch_pdl(k_lbm_adj<Real, LAT, true>, grid, b, 0, c.stream, a)
                     : launch_pdl(k_lbm_adj<Real, LAT>, grid, b, 0, c.stream, a);

@@ -26,6 +26,19 @@ BUILD.build()
     (481, 2, 2, 0, 39), (993, 1, 3, 0, 39), (497, 2, 2, 0, 39), (1025, 1, 3, 0, 39), (513, 2, 2, 0, 39),
     (962, 1, 3, 2, 39), (993, 1, 3, 0, 19)])
 def test_gradient_next_to_the_walls_of_wide_rows(ncx, lb_ratio, ncy, ncz, lattice):
+    check_gradient_next_to_the_walls(ncx, lb_ratio, ncy, ncz, lattice)
+
+
+@pytest.mark.parametrize("ncx,lb_ratio,ncy,ncz,lattice", [
+    (6, 1, 22, 0, 39), (7, 1, 19, 0, 39), (12, 1, 7, 2, 39), (20, 1, 13, 0, 19), (25, 1, 6, 0, 39),
+    (33, 1, 620, 0, 39), (21, 2, 310, 0, 19)])
+def test_gradient_of_whole_rows_in_a_block(ncx, lb_ratio, ncy, ncz, lattice):
+    # narrow rows go whole to a block, whose last one may have fewer (22 rows of 6 nodes: 21 and 1);
+    # rows of 33 and 42 nodes only on lattices this large
+    check_gradient_next_to_the_walls(ncx, lb_ratio, ncy, ncz, lattice)
+
+
+def check_gradient_next_to_the_walls(ncx, lb_ratio, ncy, ncz, lattice):
     cfg = W.config(ncx=ncx, ncy=ncy, ncz=ncz, ppc=1, lb_ratio=lb_ratio, real_bytes=8, lattice=lattice, kn=0.3, ma=0.5,
                    seed=3)
     h = B.Hybrid(cfg)
