@@ -89,14 +89,16 @@ __device__ __forceinline__ void packed_indices(int k, int& i, int& j, int& l) {
     l = (int)(code >> 4);
 }
 
-// DSMC2LB by one warp for `per` consecutive list entries. Lanes 0-19 read the cell's 20 sums and
-// scale them by one FP64 reciprocal of the particle count; the coefficients (one per lane, state
-// precision) are broadcast and each lane evaluates one or two populations. Nodes of one cell
-// have the same populations, so entries that follow one another in a cell (two nodes per cell and
-// axis) share the solve, which FP64 bounds (19 cycles per warp instruction and SM): the two
-// divisions run in two lanes of one sequence, and the factors 3 of the diagonal terms in one
-// multiplication.
-template <typename Real, class LAT>
+// DSMC2LB by one warp for one listed node, or with PAIRS for two where they lie in one cell (two nodes
+// per cell and axis, entries 2 k and 2 k + 1 next to each other along an axis), whose populations are
+// the same: the warp of the first entry solves and writes both, that of the second has nothing to do.
+// Pairs that lie in two cells (lists in any other order) so cost what single entries do. Lanes 0-19
+// read the cell's 20 sums and scale them by one FP64 reciprocal of the particle count; the
+// coefficients (one per lane, state precision) are broadcast and each lane evaluates one or two
+// populations. FP64 bounds the solve (19 cycles per warp instruction and SM): its two divisions run in
+// two lanes of one sequence, and the factors 3 of the diagonal terms in one multiplication. A warp
+// takes the entries first per + j, j < per, and on by stride per.
+template <typename Real, class LAT, bool PAIRS>
 __device__ __forceinline__ void d2l_entries(const MapArgs<Real>& a, int first, int stride, int per) {
     const LatXi<LAT, Real>& lt = lat_xi<LAT, Real>();
     const Real* sx = lt.x;
@@ -106,118 +108,118 @@ __device__ __forceinline__ void d2l_entries(const MapArgs<Real>& a, int first, i
     // the sample of a step that a batch's LB step is still to end
     if (a.pending && (a.pending == 1u || a.ctrl[CTRL_STEP] % a.pending == 0u)) S += 1u;
     constexpr int NH = (LAT::Q + 31) / 32;
-    for (int t0 = first * per; t0 < a.n; t0 += stride * per) {
-        int64_t have = -1;  // the cell whose populations f holds
-        bool usable = false;
-        Real f[NH];
-        for (int t = t0; t < t0 + per && t < a.n; ++t) {
-            const int32_t node = a.list[t];
-            if (node < 0 || (int64_t)node >= a.nnodes) {
-                if (lane == 0) atomicOr(&a.ctrl[CTRL_STATUS], HYB_ST_BAD_INPUT);
-                continue;
-            }
-            // node (z ny + y) nx + x lies in cell (iz ncy + iy) ncx + ix (z = 0 in 2D); a slab's
-            // ghost rows (the yh rows below and above its own) belong to no cell of the context
-            const int x = node % a.nx, y = (node / a.nx) % a.ny - a.yh, z = node / (a.nx * a.ny);
-            if (y < 0 || y >= a.ncy * a.lb_ratio) {
-                if (lane == 0) atomicOr(&a.ctrl[CTRL_STATUS], HYB_ST_BAD_INPUT);
-                continue;
-            }
-            const int64_t cell =
-                ((int64_t)(z / a.lb_ratio) * a.ncy + y / a.lb_ratio) * a.ncx + (x / a.lb_ratio);
-            if (cell != have) {
-                have = cell;
-                const double* m = a.acc + cell * kMoments;
-                const double mk = lane < (unsigned)kMoments ? m[lane] : 0.0;
-                const double NS = __shfl_sync(kFull, mk, 0);
-                usable = S != 0 && NS > 0.0;
-                if (usable) {
-                    // per-particle moments, lane k: <v> (1-3), <vv> (4-9), <vvv> (10-19), and the
-                    // raw Hermite coefficients, in FP64; lane 0 forms the reciprocal of the count and
-                    // lane 1 the density
-                    double qd = 0.0;
-                    if (lane < 2u) {
-                        const double SP = (double)((unsigned long long)S * (unsigned)a.ppc);
-                        qd = (lane == 0 ? 1.0 : NS) / (lane == 0 ? NS : SP);
-                    }
-                    const double inv = __shfl_sync(kFull, qd, 0), rho = __shfl_sync(kFull, qd, 1);
-                    const double mr = mk * inv;
-                    const double m1x = __shfl_sync(kFull, mr, 1);
-                    const double m1y = __shfl_sync(kFull, mr, 2);
-                    const double m1z = __shfl_sync(kFull, mr, 3);
-                    // what the coefficient subtracts: xx yy zz 1; xxx 3x, xxy y, xxz z, xyy x, xzz x,
-                    // yyy 3y, yyz z, yzz y, zzz 3z
-                    double sub = 0.0;
-                    if (lane == 4u || lane == 7u || lane == 9u) sub = 1.0;
-                    if (lane == 10u || lane == 13u || lane == 15u) sub = m1x;
-                    if (lane == 11u || lane == 16u || lane == 18u) sub = m1y;
-                    if (lane == 12u || lane == 17u || lane == 19u) sub = m1z;
-                    sub = sub * (lane == 10u || lane == 16u || lane == 19u ? 3.0 : 1.0);
-                    double coef = lane == 0 ? rho : rho * (mr - sub);
-                    if (a.eq_mode && lane >= 4u && lane < (unsigned)kMoments) {
-                        // the local equilibrium of rho and u (Sec. 4, Eq. feq_dsmc): a2 = rho u u,
-                        // a3 = rho u u u
-                        int i, j, l;
-                        packed_indices((int)lane, i, j, l);
-                        auto uu = [&](int e) { return e == 0 ? m1x : (e == 1 ? m1y : m1z); };
-                        coef = rho * uu(i) * uu(j);
-                        if (lane >= 10u) coef = coef * uu(l);
-                    }
-                    const Real coef_r = (Real)coef;
-                    Real cf[kMoments];
+    auto entry = [&](int t) {
+        const int32_t node = a.list[t];
+        const int32_t other = PAIRS && (t ^ 1) < a.n ? a.list[t ^ 1] : -1;
+        if (node < 0 || (int64_t)node >= a.nnodes) {
+            if (lane == 0) atomicOr(&a.ctrl[CTRL_STATUS], HYB_ST_BAD_INPUT);
+            return;
+        }
+        // node (z ny + y) nx + x lies in cell (iz ncy + iy) ncx + ix (z = 0 in 2D); a slab's
+        // ghost rows (the yh rows below and above its own) belong to no cell of the context
+        const int x = node % a.nx, y = (node / a.nx) % a.ny - a.yh, z = node / (a.nx * a.ny);
+        if (y < 0 || y >= a.ncy * a.lb_ratio) {
+            if (lane == 0) atomicOr(&a.ctrl[CTRL_STATUS], HYB_ST_BAD_INPUT);
+            return;
+        }
+        bool both = false;
+        if constexpr (PAIRS) {
+            // the other entry is the cell's other node along an axis: up from an even coordinate of the
+            // first entry's node, down from an odd one of the second's, so a valid node (2D has no z)
+            const int up = t & 1 ? -1 : 1;
+            both = (((x ^ t) & 1) == 0 && other == node + up) || (((y ^ t) & 1) == 0 && other == node + up * a.nx) ||
+                   (a.ncz > 0 && ((z ^ t) & 1) == 0 && other == node + up * a.nx * a.ny);
+            if (both && (t & 1)) return;
+        }
+        const int64_t cell = ((int64_t)(z / a.lb_ratio) * a.ncy + y / a.lb_ratio) * a.ncx + (x / a.lb_ratio);
+        const double* m = a.acc + cell * kMoments;
+        const double mk = lane < (unsigned)kMoments ? m[lane] : 0.0;
+        const double NS = __shfl_sync(kFull, mk, 0);
+        if (S == 0 || !(NS > 0.0)) {
+            if (lane == 0) atomicOr(&a.ctrl[CTRL_STATUS], HYB_ST_BAD_INPUT);
+            return;
+        }
+        // per-particle moments, lane k: <v> (1-3), <vv> (4-9), <vvv> (10-19), and the
+        // raw Hermite coefficients, in FP64; lane 0 forms the reciprocal of the count and
+        // lane 1 the density
+        double qd = 0.0;
+        if (lane < 2u) {
+            const double SP = (double)((unsigned long long)S * (unsigned)a.ppc);
+            qd = (lane == 0 ? 1.0 : NS) / (lane == 0 ? NS : SP);
+        }
+        const double inv = __shfl_sync(kFull, qd, 0), rho = __shfl_sync(kFull, qd, 1);
+        const double mr = mk * inv;
+        const double m1x = __shfl_sync(kFull, mr, 1);
+        const double m1y = __shfl_sync(kFull, mr, 2);
+        const double m1z = __shfl_sync(kFull, mr, 3);
+        // what the coefficient subtracts: xx yy zz 1; xxx 3x, xxy y, xxz z, xyy x, xzz x,
+        // yyy 3y, yyz z, yzz y, zzz 3z
+        double sub = 0.0;
+        if (lane == 4u || lane == 7u || lane == 9u) sub = 1.0;
+        if (lane == 10u || lane == 13u || lane == 15u) sub = m1x;
+        if (lane == 11u || lane == 16u || lane == 18u) sub = m1y;
+        if (lane == 12u || lane == 17u || lane == 19u) sub = m1z;
+        sub = sub * (lane == 10u || lane == 16u || lane == 19u ? 3.0 : 1.0);
+        double coef = lane == 0 ? rho : rho * (mr - sub);
+        if (a.eq_mode && lane >= 4u && lane < (unsigned)kMoments) {
+            // the local equilibrium of rho and u (Sec. 4, Eq. feq_dsmc): a2 = rho u u,
+            // a3 = rho u u u
+            int i, j, l;
+            packed_indices((int)lane, i, j, l);
+            auto uu = [&](int e) { return e == 0 ? m1x : (e == 1 ? m1y : m1z); };
+            coef = rho * uu(i) * uu(j);
+            if (lane >= 10u) coef = coef * uu(l);
+        }
+        const Real coef_r = (Real)coef;
+        Real cf[kMoments];
 #pragma unroll
-                    for (int k = 0; k < kMoments; ++k) cf[k] = __shfl_sync(kFull, coef_r, k);
-                    const Real* a2 = cf + 4;
-                    const Real* a3 = cf + 10;
-                    const Real tx = a3[0] + a3[3] + a3[5], ty = a3[1] + a3[6] + a3[8], tz = a3[2] + a3[7] + a3[9];
-                    const Real tr2 = a2[0] + a2[3] + a2[5];
+        for (int k = 0; k < kMoments; ++k) cf[k] = __shfl_sync(kFull, coef_r, k);
+        const Real* a2 = cf + 4;
+        const Real* a3 = cf + 10;
+        const Real tx = a3[0] + a3[3] + a3[5], ty = a3[1] + a3[6] + a3[8], tz = a3[2] + a3[7] + a3[9];
+        const Real tr2 = a2[0] + a2[3] + a2[5];
 #pragma unroll
-                    for (int h = 0; h < NH; ++h) {
-                        const int q = (int)lane + 32 * h;
-                        if (q < LAT::Q) {
-                            const Real X = sx[3 * q], Y = sx[3 * q + 1], Z = sx[3 * q + 2];
-                            const Real h2 = a2[0] * X * X + a2[3] * Y * Y + a2[5] * Z * Z - tr2 +
-                                            (Real)2 * (a2[1] * X * Y + a2[2] * X * Z + a2[4] * Y * Z);
-                            Real sum = cf[0] + cf[1] * X + cf[2] * Y + cf[3] * Z + (Real)0.5 * h2;
-                            if (LAT::ORDER >= 3) {
-                                const Real cubic = a3[0] * X * X * X + (Real)3 * a3[1] * X * X * Y +
-                                                   (Real)3 * a3[2] * X * X * Z + (Real)3 * a3[3] * X * Y * Y +
-                                                   (Real)6 * a3[4] * X * Y * Z + (Real)3 * a3[5] * X * Z * Z +
-                                                   a3[6] * Y * Y * Y + (Real)3 * a3[7] * Y * Y * Z +
-                                                   (Real)3 * a3[8] * Y * Z * Z + a3[9] * Z * Z * Z;
-                                sum += (cubic - (Real)3 * (tx * X + ty * Y + tz * Z)) * (Real)(1.0 / 6.0);
-                            }
-                            f[h] = sw[q] * sum;
-                        }
-                    }
+        for (int h = 0; h < NH; ++h) {
+            const int q = (int)lane + 32 * h;
+            if (q < LAT::Q) {
+                const Real X = sx[3 * q], Y = sx[3 * q + 1], Z = sx[3 * q + 2];
+                const Real h2 = a2[0] * X * X + a2[3] * Y * Y + a2[5] * Z * Z - tr2 +
+                                (Real)2 * (a2[1] * X * Y + a2[2] * X * Z + a2[4] * Y * Z);
+                Real sum = cf[0] + cf[1] * X + cf[2] * Y + cf[3] * Z + (Real)0.5 * h2;
+                if (LAT::ORDER >= 3) {
+                    const Real cubic = a3[0] * X * X * X + (Real)3 * a3[1] * X * X * Y +
+                                       (Real)3 * a3[2] * X * X * Z + (Real)3 * a3[3] * X * Y * Y +
+                                       (Real)6 * a3[4] * X * Y * Z + (Real)3 * a3[5] * X * Z * Z +
+                                       a3[6] * Y * Y * Y + (Real)3 * a3[7] * Y * Y * Z +
+                                       (Real)3 * a3[8] * Y * Z * Z + a3[9] * Z * Z * Z;
+                    sum += (cubic - (Real)3 * (tx * X + ty * Y + tz * Z)) * (Real)(1.0 / 6.0);
                 }
-            }
-            if (!usable) {
-                if (lane == 0) atomicOr(&a.ctrl[CTRL_STATUS], HYB_ST_BAD_INPUT);
-                continue;
-            }
-#pragma unroll
-            for (int h = 0; h < NH; ++h) {
-                const int q = (int)lane + 32 * h;
-                if (q < LAT::Q) a.f[(int64_t)q * a.nnodes + node] = f[h];
+                const Real fq = sw[q] * sum;
+                a.f[(int64_t)q * a.nnodes + node] = fq;
+                if (both) a.f[(int64_t)q * a.nnodes + other] = fq;
             }
         }
-    }
+    };
+    for (int t0 = first * per; t0 < a.n; t0 += stride * per)
+        for (int t = t0; t < t0 + per && t < a.n; ++t) entry(t);
 }
 
-// DSMC2LB: one warp per lb_ratio listed nodes, or per listed node of all replicas in the batch
-// form.
-template <typename Real, class LAT, bool BATCH>
-__global__ void __launch_bounds__(256) k_d2l(Launch<MapArgs<Real>> L) {
-    pdl_begin();
+// DSMC2LB (the listed nodes of all replicas, one per warp, in the batch form). ahead: the next kernel's
+// blocks may be placed while this one runs.
+template <typename Real, class LAT, bool BATCH, bool PAIRS = false>
+__global__ void __launch_bounds__(256) k_d2l(Launch<MapArgs<Real>> L, int per, bool ahead) {
+    if (BATCH || ahead)
+        pdl_begin();
+    else
+        pdl_after_wait(false);
     const int64_t gw = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     if constexpr (BATCH) {
         if (gw >= L.total) return;
         const int r = replica_of(L.pre, L.nrep, gw);
         const MapArgs<Real>& a = L.tab[r];
-        d2l_entries<Real, LAT>(a, (int)(gw - L.pre[r]), a.n, 1);
+        d2l_entries<Real, LAT, false>(a, (int)(gw - L.pre[r]), a.n, 1);
     } else {
-        d2l_entries<Real, LAT>(L.one, (int)gw, (int)(((int64_t)gridDim.x * blockDim.x) >> 5), L.one.lb_ratio);
+        d2l_entries<Real, LAT, PAIRS>(L.one, (int)gw, (int)(((int64_t)gridDim.x * blockDim.x) >> 5), per);
     }
 }
 
@@ -842,9 +844,21 @@ cudaError_t d2l_impl(Ctx& c, const int32_t* nodes, int32_t n) {
     Launch<MapArgs<Real>> L{};
     L.one = a;
     L.total = n;
-    const cudaError_t e = launch_pdl(k_d2l<Real, LAT, false>,
-                                     dim3(blocks_for(c, ((int64_t)n + a.lb_ratio - 1) / a.lb_ratio * 32, 128, 16)),
-                                     dim3(128), 0, c.stream, L);
+    // Pairs where an SM has several entries to solve: at 64 or 256 nodes, a lattice row's or shuffled, all
+    // are solved at once either way, and the pairs' checks cost 0.2 us of 3.0 (FP32) to 9 (FP64). At
+    // 1024 nodes and more rows of pairs take, D3Q39, FP32 3.1 us (single entries 3.4) and FP64 9.0
+    // (15.3), shuffled ones as long as single entries. Lists that fill the GPU with warps more than
+    // once have a warp take both entries (16384 nodes in rows: 11.6 us, a warp each 13.0).
+    const bool pairs = a.lb_ratio == 2 && n > 6 * c.num_sms;
+    const int per = pairs && n > 64 * c.num_sms ? 2 : 1;
+    // Blocks of the next kernel that are placed early crowd on the SMs that have room first, and on long
+    // lists and in FP64 that costs more than the overlap gives: D3Q39, one mapping after another, FP32
+    // 1024 nodes 3.1 us each against 3.6, FP64 9.1 against 18.2; the 819k-particle channel's step 54.5 us
+    // against 57.6.
+    const bool ahead = sizeof(Real) == 4 && n <= 6 * c.num_sms;
+    const dim3 grid(blocks_for(c, ((int64_t)n + per - 1) / per * 32, 64, 32)), block(64);
+    const cudaError_t e = pairs ? launch_pdl(k_d2l<Real, LAT, false, true>, grid, block, 0, c.stream, L, per, ahead)
+                                : launch_pdl(k_d2l<Real, LAT, false>, grid, block, 0, c.stream, L, per, ahead);
     prof_end(c, K_D2L);
     return e;
 }
@@ -1040,7 +1054,7 @@ cudaError_t batch_d2l_impl(BatchDev& b, int cur_p, int cur_f) {
     L.nrep = b.nrep;
     L.total = b.tot_d2l;
     const int64_t blocks = (b.tot_d2l * 32 + b.d2l_block - 1) / b.d2l_block;
-    return launch_pdl(k_d2l<Real, LAT, true>, dim3((unsigned)blocks), dim3(b.d2l_block), 0, b.stream, L);
+    return launch_pdl(k_d2l<Real, LAT, true>, dim3((unsigned)blocks), dim3(b.d2l_block), 0, b.stream, L, 1, true);
 }
 
 template <typename Real, class LAT>
