@@ -558,7 +558,7 @@ __device__ __forceinline__ MoveCtx<Real> l2d_move_ctx(const MapArgs<Real>& a) {
     return m;
 }
 
-template <typename Real, class LAT, bool Z3, bool MOVE = false>
+template <typename Real, class LAT, bool Z3, bool MOVE, bool EARLY>
 __device__ __forceinline__ void l2d_cells(const MapArgs<Real>& a, int first, int stride, const double* basis) {
     __shared__ unsigned s_am[kL2DWarps], s_em[kL2DWarps], s_vm[kL2DWarps];
     __shared__ Real s_c[20];
@@ -596,9 +596,11 @@ __device__ __forceinline__ void l2d_cells(const MapArgs<Real>& a, int first, int
         double mine = 0.0, rho = 0.0;
         uint32_t new_count = 0;
         const double ur = w == 0 ? u01d(draw(a.seed, gcell, t_step, TAG_L2D_ROUND, 0, 0).x) : 0.0;
-        // the block; results in warp 0. The first trials are drawn while the populations come in
-        grad_coefficients<Real, LAT, Z3>(a, icell, basis, ur, [&]() { draw_trial(threadIdx.x); }, mine, rho,
-                                         new_count);
+        // the block; results in warp 0. EARLY: the first trials are drawn while the populations come in
+        auto draw_first = [&]() {
+            if (EARLY) draw_trial(threadIdx.x);
+        };
+        grad_coefficients<Real, LAT, Z3>(a, icell, basis, ur, draw_first, mine, rho, new_count);
         if (w == 0) {
             GradRec& g = a.grad[ci];
             if (lane < 20u) {
@@ -665,7 +667,7 @@ __device__ __forceinline__ void l2d_cells(const MapArgs<Real>& a, int first, int
             const bool valid = j < cap;
             bool acc = false, env = false;
             if (valid) {
-                if (j0 > 0) draw_trial(j);
+                if (!EARLY || j0 > 0) draw_trial(j);
                 const Real G = grad_G<Real, LAT::ORDER>(a2, a3, X, Y, Z);
                 const Real R = (Real)u01f(r2.x);
                 env = G > C;
@@ -779,13 +781,11 @@ __device__ __forceinline__ void l2d_cells(const MapArgs<Real>& a, int first, int
     if (lane == 0 && flags) atomicOr(&a.ctrl[CTRL_STATUS], flags);
 }
 
-// LB2DSMC: one block per listed cell (the listed cells of all replicas in the batch form). MB: blocks
-// an SM is to hold. Long lists are bound by how many cells an SM has in its FP64 solve at once:
-// 4 blocks in FP32 (2048 cells in 3D, 20 hybrid steps: 8.43 ms, with 3 or 2 blocks 8.51 or
-// 8.80 ms); lists of up to two cells per SM by one cell's latency: 2 blocks, which keep the
-// registers (256 cells, 20 steps: 1.254 ms, with 3 or 4 blocks 1.269 or 1.287 ms).
-template <typename Real, class LAT, bool BATCH, bool Z3 = false, bool MOVE = false, int MB = 2>
-__global__ void __launch_bounds__(kL2DWarps * 32, sizeof(Real) == 4 ? MB : 1) k_l2d(Launch<MapArgs<Real>> L) {
+// LB2DSMC: one block per listed cell (the listed cells of all replicas in the batch form). MB: blocks an
+// SM is to hold; EARLY: a cell's first trials are drawn before its solve (l2d_launch).
+template <typename Real, class LAT, bool BATCH, bool Z3 = false, bool MOVE = false, int MB = sizeof(Real) == 4 ? 2 : 1,
+          bool EARLY = true>
+__global__ void __launch_bounds__(kL2DWarps * 32, MB) k_l2d(Launch<MapArgs<Real>> L) {
     // the basis does not depend on the previous kernel: it is fetched while that one finishes
     __shared__ double s_basis[LAT::Q * kMoments];
     for (int i = threadIdx.x; i < LAT::Q * kMoments; i += kL2DWarps * 32)
@@ -795,9 +795,9 @@ __global__ void __launch_bounds__(kL2DWarps * 32, sizeof(Real) == 4 ? MB : 1) k_
     if constexpr (BATCH) {
         const int r = replica_of(L.pre, L.nrep, (int64_t)blockIdx.x);
         const MapArgs<Real>& a = L.tab[r];
-        l2d_cells<Real, LAT, Z3, MOVE>(a, (int)(blockIdx.x - L.pre[r]), a.n, s_basis);
+        l2d_cells<Real, LAT, Z3, MOVE, EARLY>(a, (int)(blockIdx.x - L.pre[r]), a.n, s_basis);
     } else {
-        l2d_cells<Real, LAT, Z3, MOVE>(L.one, (int)blockIdx.x, (int)gridDim.x, s_basis);
+        l2d_cells<Real, LAT, Z3, MOVE, EARLY>(L.one, (int)blockIdx.x, (int)gridDim.x, s_basis);
     }
 }
 
@@ -870,15 +870,40 @@ cudaError_t l2d_launch(Ctx& c, const MapArgs<Real>& a, int32_t n) {
     L.one = a;
     L.total = n;
     const dim3 grid(blocks_for(c, (int64_t)n * 32 * kL2DWarps, 32 * kL2DWarps, 8)), block(32 * kL2DWarps);
-    constexpr int LONG = sizeof(Real) == 4 ? 4 : 2;  // (in FP64 the same kernel)
-    const bool longer = n > 2 * c.num_sms;
+    // Blocks per SM. Lists that one block per SM (FP64) or two (FP32) take at once are bound by one
+    // cell's latency, and more blocks cost registers; longer ones by how many cells an SM has in its
+    // solve and its trials at once. us a mapping, one after another, of n cells:
+    //   FP64  D3Q39 152 cells 23.2 with one block, 23.0 with two; 256 45.3 / 40.4; 1024 155.8 / 135.3;
+    //         D3Q19 256 34.7 / 31.2, 1024 119 / 102. (Where most first trials are rejected, as after four
+    //         samples, one block is faster up to four cells per SM: 256 cells of D3Q39 130 / 149.)
+    //   FP32  D3Q39 304 cells with two blocks 7.6, with four 7.4; 305 13.5 / 9.0; 4096 87 / 54 (five: 57);
+    //         D3Q19 304 6.3 / 6.2; 608 11.8 / 7.7; 4096 67 / 42.8, with five blocks 40.7: five where
+    //         they take fewer rounds than four, 760 cells 9.4 against 12.6, 1024 13.7 against 13.6.
+    // The first trials come early but for D3Q19 with as many blocks as the registers give, where other
+    // cells hide the loads and the draws' registers spill (4096 cells, FP64 403 against 382 us).
+    auto launch = [&](auto mb, auto early) {
+        constexpr int MB = decltype(mb)::value;
+        constexpr bool EARLY = decltype(early)::value;
+        return a.ncz ? launch_pdl(k_l2d<Real, LAT, false, true, MOVE, MB, EARLY>, grid, block, 0, c.stream, L)
+                     : launch_pdl(k_l2d<Real, LAT, false, false, MOVE, MB, EARLY>, grid, block, 0, c.stream, L);
+    };
+    using std::integral_constant;
+    constexpr integral_constant<bool, true> early;
+    const int sms = c.num_sms;
     cudaError_t e;
-    if (a.ncz)
-        e = longer ? launch_pdl(k_l2d<Real, LAT, false, true, MOVE, LONG>, grid, block, 0, c.stream, L)
-                   : launch_pdl(k_l2d<Real, LAT, false, true, MOVE>, grid, block, 0, c.stream, L);
-    else
-        e = longer ? launch_pdl(k_l2d<Real, LAT, false, false, MOVE, LONG>, grid, block, 0, c.stream, L)
-                   : launch_pdl(k_l2d<Real, LAT, false, false, MOVE>, grid, block, 0, c.stream, L);
+    if constexpr (sizeof(Real) == 8) {
+        e = n <= sms ? launch(integral_constant<int, 1>(), early)
+                     : launch(integral_constant<int, 2>(), integral_constant<bool, LAT::Q == 39>());
+    } else if (n <= 2 * sms) {
+        e = launch(integral_constant<int, 2>(), early);
+    } else {
+        // (the fused pass's LB2DSMC, which moves the particles on, needs the registers)
+        constexpr bool FIVE = LAT::Q == 19 && !MOVE;
+        if (FIVE && (n + 5 * sms - 1) / (5 * sms) < (n + 4 * sms - 1) / (4 * sms))
+            e = launch(integral_constant<int, FIVE ? 5 : 4>(), integral_constant<bool, !FIVE>());
+        else
+            e = launch(integral_constant<int, 4>(), early);
+    }
     prof_end(c, K_L2D);
     return e;
 }
