@@ -156,8 +156,10 @@ __device__ __forceinline__ Half<Real> half_d(const DsmcArgs<Real>& a) {
 // square root, sine and cosine), and a warp would spend them again for every 32 particles of
 // which one hits: such particles are listed in `later` and taken together, packed, when the others
 // are done (20 steps of the FP64 64-cell channel 3.03 -> 2.80 ms, of 64 x 64 cells
-// 3.52 -> 3.32 ms). In FP32 the list cost what it saved (64 batched channels, 10 steps:
-// 1.11 against 1.04 ms).
+// 3.52 -> 3.32 ms). A cell of at most 32 particles takes them all in one trip, wall or not: with a
+// second trip for the walls' the move of 16k cells of 8 particles took 43.2 us, in 3D 60.4, against
+// 38.3 and 53.6 in one. In FP32 the list cost what it saved (64 batched channels, 10
+// steps: 1.11 against 1.04 ms).
 template <typename Real, bool Z3>
 __device__ __forceinline__ void move_cell(const DsmcArgs<Real>& a, int c, unsigned lane, uint8_t* later) {
     const uint32_t s = a.ctrl[CTRL_STEP];
@@ -188,6 +190,9 @@ __device__ __forceinline__ void move_cell(const DsmcArgs<Real>& a, int c, unsign
                                     p[5], lost);
         }
     };
+    // all of a cell's particles in one trip of the warp: nothing to pack
+    const bool few = PACK && n <= 32;
+    Real p0[6] = {0, 0, 0, 0, 0, 0};
     for (uint32_t k0 = 0; k0 == 0 || k0 < n; k0 += 64) {
         const uint32_t k1 = k0 + lane, k2 = k1 + 32;
         Real p1[6] = {0, 0, 0, 0, 0, 0}, p2[6] = {0, 0, 0, 0, 0, 0};  // x y z vx vy vz
@@ -195,6 +200,11 @@ __device__ __forceinline__ void move_cell(const DsmcArgs<Real>& a, int c, unsign
         // the loads need only the bin size, not the count, so they travel with it
         if (k1 < bin) rec_get(src, base + k1, p1[0], p1[1], p1[2], p1[3], p1[4], p1[5], t1);
         if (k2 < bin) rec_get(src, base + k2, p2[0], p2[1], p2[2], p2[3], p2[4], p2[5], t2);
+        if (few) {
+#pragma unroll
+            for (int i = 0; i < 6; ++i) p0[i] = p1[i];
+            break;
+        }
         const bool act1 = k1 < n && (!PACK || flies_straight(m, p1[0], p1[3]));
         const bool act2 = k2 < n && (!PACK || flies_straight(m, p2[0], p2[3]));
         if constexpr (PACK) {
@@ -217,16 +227,17 @@ __device__ __forceinline__ void move_cell(const DsmcArgs<Real>& a, int c, unsign
         put_away(act1, dir1, key1, arr1, ok1, p1);
         put_away(act2, dir2, key2, arr2, ok2, p2);
     }
+    if (few) nlater = n;
     if (PACK && nlater > 0) {
         __syncwarp();
         for (uint32_t i0 = 0; i0 < nlater; i0 += 32) {
             const bool act = i0 + lane < nlater;
-            Real p[6] = {0, 0, 0, 0, 0, 0};
+            Real p[6] = {p0[0], p0[1], p0[2], p0[3], p0[4], p0[5]};
             uint32_t key = 0, ok = 0, t;
             int dir = -1;
             if (act) {
-                const uint32_t k = later[i0 + lane];
-                rec_get(src, base + k, p[0], p[1], p[2], p[3], p[4], p[5], t);
+                const uint32_t k = few ? lane : later[i0 + lane];
+                if (!few) rec_get(src, base + k, p[0], p[1], p[2], p[3], p[4], p[5], t);
                 key = move_particle<Real, Z3>(m, org, k, s, p[0], p[1], p[2], p[3], p[4], p[5], hits, caps, dir, ok);
             }
             const uint32_t arr = bin_arrival1(dst.count, key, act && dir < 0, lane);
