@@ -878,12 +878,14 @@ LbmArgs<Real> lbm_args(const Ctx& c, int cur_f) {
 // than others: us per step with 32 / 128 threads, FP32 slab: D3Q39 65k nodes 7.98 / 9.15, 131k
 // 8.77 / 9.41, 154k 8.82 / 9.49, 197k 10.86 / 10.99, 262k 13.64 / 13.51, 8k 4.13 / 4.40, 64 nodes
 // 3.25 / 2.90; D3Q19 65k 4.08 / 6.07, 131k 5.93 / 5.72. In 3D (65k nodes 7.50 / 6.49) and FP64 (65k
-// nodes 139 / 137) the larger blocks are faster.
+// nodes 139 / 137) the larger blocks are faster, and on streamwise slabs, whose step comes between
+// the ghost rows' kernels of all slabs (two slabs of 66k nodes, exchange and step 52.2 / 48.2, of 82k
+// 51.5 / 49.7, four of 17k 94.8 / 93.6).
 template <typename Real, class LAT>
 unsigned lbm_block(const Ctx& c) {
     const int64_t most = (int64_t)c.num_sms * 32 * (LAT::Q == 39 ? 32 : 16);
     const bool one_wave = c.d.nnodes >= (int64_t)c.num_sms * 32 && c.d.nnodes <= most;
-    return sizeof(Real) == 4 && c.d.nz == 1 && one_wave ? 32u : 128u;
+    return sizeof(Real) == 4 && c.d.nz == 1 && c.d.yh == 0 && one_wave ? 32u : 128u;
 }
 
 template <typename Real, class LAT>
