@@ -844,19 +844,23 @@ cudaError_t d2l_impl(Ctx& c, const int32_t* nodes, int32_t n) {
     Launch<MapArgs<Real>> L{};
     L.one = a;
     L.total = n;
-    // Pairs where an SM has several entries to solve: at 64 or 256 nodes, a lattice row's or shuffled, all
-    // are solved at once either way, and the pairs' checks cost 0.2 us of 3.0 (FP32) to 9 (FP64). At
-    // 1024 nodes and more rows of pairs take, D3Q39, FP32 3.1 us (single entries 3.4) and FP64 9.0
-    // (15.3), shuffled ones as long as single entries. Lists that fill the GPU with warps more than
-    // once have a warp take both entries (16384 nodes in rows: 11.6 us, a warp each 13.0).
-    const bool pairs = a.lb_ratio == 2 && n > 6 * c.num_sms;
+    // Two nodes per cell and axis: a pair a warp, or two warps of which one has nothing to do; a warp for
+    // both where the list would fill the GPU with warps more than once (16384 nodes in rows: 11.5 us, a
+    // warp each 13.0). Lists in rows, D3Q39, us for 64 / 1024 / 4096 nodes: FP32 2.8 / 3.0 / 4.6, shuffled
+    // 2.9 / 3.5 / 6.2, every entry by itself 2.8 / 3.4 / 6.1; FP64 7.9 / 9.0 / 29, 7.9 / 15.3 / 49, 7.8 /
+    // 15.1 / 49.
+    const bool pairs = a.lb_ratio == 2;
     const int per = pairs && n > 64 * c.num_sms ? 2 : 1;
+    // blocks of four warps; FP64 of two, which spread its solves more evenly (4096 nodes in rows 29 us, in
+    // blocks of four 35)
+    constexpr int BLOCK = sizeof(Real) == 4 ? 128 : 64;
     // Blocks of the next kernel that are placed early crowd on the SMs that have room first, and on long
     // lists and in FP64 that costs more than the overlap gives: D3Q39, one mapping after another, FP32
     // 1024 nodes 3.1 us each against 3.6, FP64 9.1 against 18.2; the 819k-particle channel's step 54.5 us
-    // against 57.6.
-    const bool ahead = sizeof(Real) == 4 && n <= 6 * c.num_sms;
-    const dim3 grid(blocks_for(c, ((int64_t)n + per - 1) / per * 32, 64, 32)), block(64);
+    // against 57.6. (Lists that fill the GPU leave no room to crowd in: a 157 x 4 x 2 channel's step 72.2 us
+    // with the overlap, 73.2 without.)
+    const bool ahead = sizeof(Real) == 4 && (n <= 6 * c.num_sms || per == 2);
+    const dim3 grid(blocks_for(c, ((int64_t)n + per - 1) / per * 32, BLOCK, 2048 / BLOCK)), block(BLOCK);
     const cudaError_t e = pairs ? launch_pdl(k_d2l<Real, LAT, false, true>, grid, block, 0, c.stream, L, per, ahead)
                                 : launch_pdl(k_d2l<Real, LAT, false>, grid, block, 0, c.stream, L, per, ahead);
     prof_end(c, K_D2L);
@@ -879,6 +883,7 @@ cudaError_t l2d_launch(Ctx& c, const MapArgs<Real>& a, int32_t n) {
     //   FP32  D3Q39 304 cells with two blocks 7.6, with four 7.4; 305 13.5 / 9.0; 4096 87 / 54 (five: 57);
     //         D3Q19 304 6.3 / 6.2; 608 11.8 / 7.7; 4096 67 / 42.8, with five blocks 40.7: five where
     //         they take fewer rounds than four, 760 cells 9.4 against 12.6, 1024 13.7 against 13.6.
+    // Four FP32 blocks of D3Q39 that move the particles on spill 48 bytes (3D 72).
     // The first trials come early but for D3Q19 with as many blocks as the registers give, where other
     // cells hide the loads and the draws' registers spill (4096 cells, FP64 403 against 382 us).
     auto launch = [&](auto mb, auto early) {

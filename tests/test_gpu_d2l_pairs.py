@@ -1,7 +1,7 @@
-"""DSMC2LB of long lists takes two entries of one cell together where they are neighbours along an axis:
-lists in rows, shifted by one, along the other axes, shuffled, of odd length, with repeated nodes and
-with indices out of range (among them the one that would be the neighbour above a 2D lattice) give
-every node exactly the populations that short lists, which take every entry by itself, give."""
+"""DSMC2LB takes two entries of one cell together where they are neighbours along an axis: lists in rows,
+shifted by one, along the other axes, shuffled, of odd length, with repeated nodes and with indices out
+of range (among them the one that would be the neighbour above a 2D lattice), of fewer and of more
+entries than the GPU has warps, give every node exactly the populations that lists of one entry give."""
 import numpy as np
 import pytest
 
@@ -17,8 +17,6 @@ from paper_1512_08042_gb300 import binding as B  # noqa: E402
 from paper_1512_08042_gb300 import build as BUILD  # noqa: E402
 
 BUILD.build()
-
-SHORT = 500  # entries by themselves
 
 
 def _order(nodes, nx, plane, order):
@@ -45,18 +43,17 @@ def _order(nodes, nx, plane, order):
     (4, 39, 0, 20, 30, 2), (8, 39, 0, 20, 30, 2), (4, 19, 4, 10, 12, 2), (8, 19, 3, 7, 13, 2), (4, 39, 0, 64, 60, 2),
     (4, 39, 0, 40, 40, 1)])
 @pytest.mark.parametrize("order", ["rows", "shifted", "columns", "layers", "shuffled", "odd"])
-def test_long_lists_equal_short_ones(real_bytes, lattice, ncz, ncx, ncy, lb_ratio, order):
+def test_lists_equal_single_entries(real_bytes, lattice, ncz, ncx, ncy, lb_ratio, order):
     cfg = W.config(ncx=ncx, ncy=ncy, ncz=ncz, ppc=20, lb_ratio=lb_ratio, real_bytes=real_bytes, lattice=lattice, seed=4)
     a, b = B.Hybrid(cfg), B.Hybrid(cfg)
     for h in (a, b):
         h.dsmc_step(2)
     nx, ny, nn = int(a.d["nx"]), int(a.d["ny"]), int(a.d["nnodes"])
-    assert nn > 6 * 200
     nodes = _order(np.arange(nn, dtype=np.int32), nx, nx * ny, order).astype(np.int32)
     dev = torch.from_numpy(np.ascontiguousarray(nodes)).cuda()
     a.map_dsmc_to_lbm(dev)
-    for k in range(0, len(nodes), SHORT):
-        b.map_dsmc_to_lbm(dev[k:k + SHORT])
+    for k in range(len(nodes)):
+        b.map_dsmc_to_lbm(dev[k:k + 1])
     assert a.sync_status() == b.sync_status()
     assert bool(a.sync_status()[1] & B.ST_BAD_INPUT) == (order == "odd")
     assert torch.equal(a.f(), b.f())
@@ -64,7 +61,7 @@ def test_long_lists_equal_short_ones(real_bytes, lattice, ncz, ncx, ncy, lb_rati
     b.close()
 
 
-def test_long_lists_of_a_slab_skip_its_ghost_rows():
+def test_lists_of_a_slab_skip_its_ghost_rows():
     cfg = W.config(ncx=24, ncy=20, ppc=20, lb_ratio=2, seed=4, ncy_global=40, y0=10)
     a, b = B.Hybrid(cfg), B.Hybrid(cfg)
     for h in (a, b):
@@ -74,8 +71,8 @@ def test_long_lists_of_a_slab_skip_its_ghost_rows():
     nodes = np.arange(int(a.d["nnodes"]), dtype=np.int32)
     dev = torch.from_numpy(nodes).cuda()
     a.map_dsmc_to_lbm(dev)
-    for k in range(0, len(nodes), SHORT):
-        b.map_dsmc_to_lbm(dev[k:k + SHORT])
+    for k in range(len(nodes)):
+        b.map_dsmc_to_lbm(dev[k:k + 1])
     assert a.sync_status() == b.sync_status() and a.sync_status()[1] & B.ST_BAD_INPUT
     assert torch.equal(a.f(), b.f())
     a.close()
