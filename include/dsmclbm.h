@@ -337,9 +337,10 @@ hyb_status lbm_interface_loss(hyb_ctx* ctx, const void* f, const int32_t* dev_no
 
 /* One step of the adjoint: with f the populations at step t and lam_next = dL/df_{t+1},
  * writes lam = dL/df_t (every entry) and adds dL/dg and dL/dtau of this step to grad_g and
- * grad_tau. wall is a scratch of 2 * ny * nz + 1 values (state precision; nz = 1 for the
- * slab) that must be zero before the first call; it is left zero. lam and lam_next must differ. The adjoint is that of the regularised
- * collision: a context with lb_collision = 1 returns HYB_EINVAL. */
+ * grad_tau. wall (2 * ny * nz + 1 values of the state precision; nz = 1 for the slab; not NULL) is
+ * kept for callers of the call's earlier form: it is neither read nor written. lam and lam_next must
+ * differ. The adjoint is that of the regularised collision: a context with lb_collision = 1 returns
+ * HYB_EINVAL. */
 hyb_status lbm_adjoint_step(hyb_ctx* ctx, const void* f, const void* lam_next, void* lam,
                             const void* g_node, const void* tau_node, void* grad_g,
                             void* grad_tau, void* wall);
@@ -436,9 +437,9 @@ hyb_status hyb_current(const hyb_ctx* ctx, int32_t* particle_half, int32_t* lb_h
 
 /* Whether dsmc_step and hyb_hybrid_step with nsteps > 1 fuse the collide of a step with the
  * move of the next (one pass over the particles per step). HYB_FUSE_AUTO (the default) fuses
- * when the fused pass's grid fills the GPU (at least as many blocks of 32 cells as are
- * resident at once), where it is faster; below that two passes per step are. The results are
- * the same bit for bit. HYB_EINVAL for another mode. */
+ * when the fused pass's grid fills the GPU (at least as many blocks of the context's collide shape as
+ * are resident at once), about where FP32 hybrid steps become faster so; hyb_tune_collide measures it
+ * for a context. The results are the same bit for bit. HYB_EINVAL for another mode. */
 #define HYB_FUSE_AUTO 0
 #define HYB_FUSE_ALWAYS 1
 #define HYB_FUSE_NEVER 2

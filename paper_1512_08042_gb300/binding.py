@@ -359,7 +359,7 @@ class Hybrid:
                self.ctx)
 
     def wall_scratch_size(self):
-        """Values of the adjoint's wall scratch: two sums per streamwise row (y, z), a ticket."""
+        """Values of the adjoint calls' `wall` argument (which they neither read nor write)."""
         return 2 * int(self.d["ny"]) * int(self.d["nz"]) + 1
 
     def map_dsmc_to_lbm_adjoint(self, nodes, lam, grad_acc):
@@ -376,7 +376,7 @@ class Hybrid:
 
     def lbm_adjoint_step(self, f, lam_next, lam, g, tau, grad_g, grad_tau, wall):
         """lam = dL/df_t from f_t and lam_next = dL/df_{t+1}; adds this step's dL/dg and
-        dL/dtau to grad_g and grad_tau. wall: 2 ny nz + 1 zeros, left zero."""
+        dL/dtau to grad_g and grad_tau. wall: 2 ny nz + 1 values, neither read nor written."""
         self._check_pop(f, lam_next, lam)
         self._check_node(g, tau, grad_g, grad_tau)
         if wall.numel() != self.wall_scratch_size() or wall.dtype != self.real:
@@ -978,7 +978,7 @@ def _loss_adjoint(h, g, tau, lam_T, ckpts, T, K):
     with torch.cuda.stream(h.stream):
         grad_g = torch.zeros_like(g)
         grad_tau = torch.zeros_like(tau)
-        wall = torch.zeros(h.wall_scratch_size(), dtype=g.dtype, device=g.device)
+        wall = torch.empty(h.wall_scratch_size(), dtype=g.dtype, device=g.device)  # untouched
         lam_next = lam_T.clone()
         lam = torch.empty_like(lam_next)
         scratch = torch.empty((max(K - 1, 1),) + tuple(lam_next.shape), dtype=lam_next.dtype,

@@ -49,12 +49,6 @@ __device__ __forceinline__ void rec_get(const double* rec, int64_t i, double& x,
     z = c.y;
     tag = (uint32_t)__double_as_longlong(d.x);
 }
-__device__ __forceinline__ uint32_t rec_tag(const float* rec, int64_t i) {
-    return __float_as_uint(rec[(int64_t)kRec * i + RS_TAG]);
-}
-__device__ __forceinline__ uint32_t rec_tag(const double* rec, int64_t i) {
-    return (uint32_t)__double_as_longlong(rec[(int64_t)kRec * i + RS_TAG]);
-}
 
 // What a move needs: channel sizes, step constants rounded to the state precision, the key.
 template <typename Real>

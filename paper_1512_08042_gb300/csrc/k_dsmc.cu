@@ -287,7 +287,8 @@ constexpr int kWarpCells = 32 / kGroup;
 // Blocks of 8 warps (32 cells) or 4 (16 cells) only group warps for a launch: a block keeps its
 // shared memory until its slowest warp is done, so 4 are faster where the grid runs many waves
 // (105M particles, 20 steps: 61.7 against 63.7 ms) and 8 by 2% where it does not. 24 resident warps
-// per SM in FP32 (80 registers): 28 took 67.2 ms (spills, and little L1 left beside the pools).
+// per SM in FP32 (80 registers; the 3D fused pass spills 32 bytes at them): 28 took 67.2 ms (spills, and
+// little L1 left beside the pools).
 constexpr int kCollideWarps = 8;
 template <typename Real, int W>
 struct CollideCfg {
@@ -1260,10 +1261,14 @@ int collide_per_sm(Kern kernel, int threads, size_t smem) {
 }
 }  // namespace
 
-// Whether the fused pass's grid fills the GPU: at least as many blocks of 32 cells as fit on
-// it at once. Below that a launch is one partial wave whose time is the latency of its
-// slowest block, which the fused pass lengthens (a collide and a move in one block), and two
-// separate passes are faster.
+// Whether the fused pass's grid fills the GPU: at least as many blocks of the context's shape as fit
+// on it at once. Below that a launch is one partial wave whose time is the latency of its slowest
+// block, which the fused pass lengthens (a collide and a move in one block). us a step of ten-step calls,
+// two passes / fused: hybrid steps 64 x 64 cells 40.6 / 42.6, 64 x 256 (just above) 53.4 / 55.7, 128 x 512
+// 153 / 128; DSMC alone 40 x 40 cells at Kn 0.02 42.8 / 34.8, 64 x 64 26.4 / 24.3, 64 x 256 35.8 / 37.9,
+// 128 x 512 124 / 97. FP64 passes are faster apart at every size measured (64 x 64 hybrid 229 / 271,
+// 64 x 256 376 / 433): the one line for both calls and precisions lies where FP32 hybrid steps change
+// over; hyb_set_fuse and the tuner choose otherwise.
 namespace {
 template <typename Real, bool Z3, int W>
 int fused_per_sm(const Ctx& c) {

@@ -875,7 +875,7 @@ LbmArgs<Real> lbm_args(const Ctx& c, int cur_f) {
 
 // Threads per block of the plain LB step. One-warp blocks spread a lattice of at most one wave
 // evenly over the SMs (an SM holds 32 blocks) where blocks of 128 leave some SMs four warps more
-// than others: us per step with 32 / 128 threads, FP32 slab: D3Q39 65k nodes 7.98 / 9.15, 131k
+// than others: us per step with 32 / 128 threads, FP32 in 2D: D3Q39 65k nodes 7.98 / 9.15, 131k
 // 8.77 / 9.41, 154k 8.82 / 9.49, 197k 10.86 / 10.99, 262k 13.64 / 13.51, 8k 4.13 / 4.40, 64 nodes
 // 3.25 / 2.90; D3Q19 65k 4.08 / 6.07, 131k 5.93 / 5.72. In 3D (65k nodes 7.50 / 6.49) and FP64 (65k
 // nodes 139 / 137) the larger blocks are faster, and on streamwise slabs, whose step comes between

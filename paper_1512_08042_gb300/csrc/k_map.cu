@@ -857,7 +857,7 @@ cudaError_t d2l_impl(Ctx& c, const int32_t* nodes, int32_t n) {
     // Blocks of the next kernel that are placed early crowd on the SMs that have room first, and on long
     // lists and in FP64 that costs more than the overlap gives: D3Q39, one mapping after another, FP32
     // 1024 nodes 3.1 us each against 3.6, FP64 9.1 against 18.2; the 819k-particle channel's step 54.5 us
-    // against 57.6. (Lists that fill the GPU leave no room to crowd in: a 157 x 4 x 2 channel's step 72.2 us
+    // against 57.6. (Lists that fill the GPU leave no room to crowd in: a 157 x 4 x 2 channel's step 71.7 us
     // with the overlap, 73.2 without.)
     const bool ahead = sizeof(Real) == 4 && (n <= 6 * c.num_sms || per == 2);
     const dim3 grid(blocks_for(c, ((int64_t)n + per - 1) / per * 32, BLOCK, 2048 / BLOCK)), block(BLOCK);
