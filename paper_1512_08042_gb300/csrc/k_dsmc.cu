@@ -1116,7 +1116,7 @@ cudaError_t move_impl(Ctx& c, int p) {
 // leave the block within the shared memory a block may have (limit), and at least one bin, which the
 // largest bins leave room for in either shape. A smaller pool only has more warps take their cells one
 // at a time. Bins of 128 to 256 slots need it: in blocks of 8 warps from 95 particles per cell on in
-// FP64 3D (at a capacity factor of 2.5), 132 in FP64 2D and 189 in FP32 3D, in blocks of 4 from 223 in
+// FP64 3D (at a capacity factor of 2.5), 130 in FP64 2D and 183 in FP32 3D, in blocks of 4 from 223 in
 // FP64 3D.
 template <typename Real, bool Z3>
 uint32_t fitting_pool(uint32_t pool, uint32_t bin, int warps, int limit) {
